@@ -98,3 +98,26 @@ def test_forces_noalloc_rejects_sizes_beyond_the_scratch():
     with pytest.raises(md.MDError) as e:
         md.md_forces_noalloc([80.0, 80.0, 80.0], 100, RC, tp.data_ptr(), tf.data_ptr(), te.data_ptr())
     assert e.value.code == md.MD_EINVAL
+
+
+# (n, rho, jitter, aspect): one atom, one block of 32 atoms and one more, the
+# 3-cell grid (every cell at a periodic face), the largest size that one block
+# bins and the next, a dense state whose atoms queue more pairs than the
+# queue holds, an elongated box, more than one scan tile of cells.
+@pytest.mark.parametrize("case", [(1, 0.02, 0.0, (1, 1, 1)), (32, 0.7, 0.1, (1, 1, 1)), (33, 0.7, 0.1, (1, 1, 1)),
+                                  (4096, 0.9, 0.1, (1, 1, 1)), (4097, 0.9, 0.1, (1.0, 1.3, 0.8)),
+                                  (500, 3.0, 0.02, (1, 1, 1)), (6000, 3.0, 0.02, (1, 1, 1)),
+                                  (3000, 0.7, 0.15, (20.0, 1.0, 1.0)), (300, 0.1, 0.3, (1, 1, 1))])
+def test_forces_noalloc_at_the_edges_of_its_kernels(case):
+    torch = pytest.importorskip("torch")
+    ensure_built()
+    n, rho, jitter, aspect = case
+    pos, vel, L = state(n, rho, 1.0, 21, jitter=jitter, aspect=aspect)
+    pw = oracle.wrap(pos, L)
+    f_ref, u_ref, w_ref = oracle.forces_cells(pw, L, oracle_grid(L, RC), RC, 1.0)
+    f, u, w = _noalloc(torch, pos, L)
+    # FP64 sums in another order: a few ulps of the largest pair force
+    scale = max(np.abs(f_ref).max(), 1.0)
+    assert np.abs(f - f_ref).max() <= 1e-12 * scale * max(1.0, n / 1000.0)
+    assert u == pytest.approx(u_ref, rel=10 * FORCE_TOL["fp64"], abs=1e-12)
+    assert w == pytest.approx(w_ref, rel=10 * FORCE_TOL["fp64"], abs=1e-12)
