@@ -30,7 +30,15 @@ using namespace md;
 
 thread_local std::string g_create_error;
 
-constexpr int kChunk = 32;  // steps per graph replay
+// Steps per graph replay.  A call's steps but the last run as replays of
+// graphs of plain steps, as many as fit of each length (whole numbers of
+// kRebuildEvery, so that no conditional node is left over, then single
+// steps); the last runs in a graph of its own, whose step kernel also writes
+// the energies.  When every graph ended in that kernel and all remaining
+// steps were single ones, 20 steps at 1M atoms in FP64 took 11.0 ms, all in
+// the energy kernel.
+constexpr int kChunks[] = {10 * kRebuildEvery, kRebuildEvery, 1};
+constexpr int kNumChunks = sizeof(kChunks) / sizeof(kChunks[0]);
 
 // Zeroed storage for cudaGraphNodeParams (its union has no default
 // constructor).
@@ -100,10 +108,8 @@ struct Sim : SimBase {
     struct Chunk {
         cudaGraph_t g = nullptr;
         cudaGraphExec_t e = nullptr;
-        int K = 0;
     };
-    Chunk big, one;
-    bool graphs_ok = false;
+    Chunk plain[kNumChunks], last;  // instantiated when first used
 
     bool profiling = false;
     std::vector<cudaEvent_t> ev;
@@ -317,15 +323,15 @@ struct Sim : SimBase {
 
     // ---- graphs ----------------------------------------------------------
 
+    void destroy_graph(Chunk& c) {
+        if (c.e) cudaGraphExecDestroy(c.e);
+        if (c.g) cudaGraphDestroy(c.g);
+        c.e = nullptr;
+        c.g = nullptr;
+    }
     void destroy_graphs() {
-        for (Chunk* c : {&big, &one}) {
-            if (c->e) cudaGraphExecDestroy(c->e);
-            if (c->g) cudaGraphDestroy(c->g);
-            c->e = nullptr;
-            c->g = nullptr;
-            c->K = 0;
-        }
-        graphs_ok = false;
+        for (Chunk& c : plain) destroy_graph(c);
+        destroy_graph(last);
     }
 
     template <class... T>
@@ -362,12 +368,13 @@ struct Sim : SimBase {
         return MD_OK;
     }
 
-    // K steps: k_cond, then per step the step kernel and its closing kernel,
+    // K steps, plain ones or (final_node, K = 1) the one that may be a call's
+    // last: k_cond, then per step the step kernel and its closing kernel,
     // with a conditional rebuild node before every m-th step (every step in
     // the cell-list-only form, which rebuilds at each).  The closing kernel
     // before a conditional node sets its handle; a step after another whose
     // rebuild is due waits for the next conditional node.
-    int build_chunk(Chunk& c, int K) {
+    int build_chunk(Chunk& c, int K, bool final_node) {
         MD_CUDA(cudaGraphCreate(&c.g, 0));
         const int m = (prm.cell_list_only || a.n > kRebuildEveryMaxAtoms) ? 1 : kRebuildEvery;
         std::vector<cudaGraphConditionalHandle> h((K + m - 1) / m);
@@ -392,30 +399,33 @@ struct Sim : SimBase {
             }
             const int has = (s + 1 < K && (s + 1) % m == 0) ? 1 : 0;
             cudaGraphConditionalHandle nxt = has ? h[(s + 1) / m] : 0;
-            // only a graph's last node can meet the last step of a call
-            MD_CUDA(add_kernel(c.g, &prev, &node, step_fn(s + 1 == K), step_grid(s + 1 == K), step_block(s + 1 == K),
+            MD_CUDA(add_kernel(c.g, &prev, &node, step_fn(final_node), step_grid(final_node), step_block(final_node),
                                a, mode, nxt, has));
             if (kStepTailNode) {
                 cudaGraphNode_t stepn = node;
-                MD_CUDA(add_kernel(c.g, &stepn, &node, tail_fn(s + 1 == K), 1, 32, a, mode, nxt, has));
+                MD_CUDA(add_kernel(c.g, &stepn, &node, tail_fn(final_node), 1, 32, a, mode, nxt, has));
             }
             prev = node;
         }
         MD_CUDA(cudaGraphInstantiate(&c.e, c.g, 0));
-        c.K = K;
         return MD_OK;
     }
 
-    int ensure_graphs() {
-        if (graphs_ok) return MD_OK;
-        destroy_graphs();
-        int r = build_chunk(big, kChunk);
-        if (!r) r = build_chunk(one, 1);
-        if (r) {
-            destroy_graphs();
-            return r;
+    // Queues `count` replays of a graph of K steps.
+    int replay(Chunk& c, int K, bool final_node, int64_t count) {
+        if (count <= 0) return MD_OK;
+        if (!c.e) {
+            int r = build_chunk(c, K, final_node);
+            if (r) {
+                destroy_graph(c);
+                return r;
+            }
         }
-        graphs_ok = true;
+        for (int64_t b = 0; b < count; b++) {
+            MD_CUDA(cudaGraphLaunch(c.e, stream));
+            graph_launches++;
+            launches += 1 + K * (kStepTailNode ? 2 : 1);
+        }
         return MD_OK;
     }
 
@@ -425,19 +435,16 @@ struct Sim : SimBase {
     int run_steps(int64_t nsteps) {
         if (nsteps <= 0) return MD_OK;
         if (prm.use_graphs && !profiling) {
-            int r = ensure_graphs();
+            // (a plain step must not meet a call's last one: steps that wait
+            // for a rebuild only leave more to run, never fewer)
+            int64_t left = nsteps - 1;
+            for (int k = 0; k < kNumChunks; k++) {
+                int r = replay(plain[k], kChunks[k], false, left / kChunks[k]);
+                if (r) return r;
+                left %= kChunks[k];
+            }
+            int r = replay(last, 1, true, 1);
             if (r) return r;
-            int64_t nb = nsteps / kChunk, rem = nsteps % kChunk;
-            for (int64_t b = 0; b < nb; b++) {
-                MD_CUDA(cudaGraphLaunch(big.e, stream));
-                graph_launches++;
-                launches += 1 + kChunk * (kStepTailNode ? 2 : 1);
-            }
-            for (int64_t b = 0; b < rem; b++) {
-                MD_CUDA(cudaGraphLaunch(one.e, stream));
-                graph_launches++;
-                launches += kStepTailNode ? 3 : 2;
-            }
         } else {
             if (profiling && (int64_t)ev.size() < 4 * nsteps) {
                 while ((int64_t)ev.size() < 4 * nsteps) {
