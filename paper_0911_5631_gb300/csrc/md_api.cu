@@ -278,7 +278,8 @@ struct Sim : SimBase {
     }
     // threads per block of the step kernel (the final step always kBlock)
     unsigned step_block(bool final_node) const {
-        if (final_node || P::kFp64 || prm.cell_list_only) return kBlock;
+        if (final_node || prm.cell_list_only) return kBlock;
+        if (P::kFp64) return kStepBlockF64;
         if (prm.variant == MD_VARIANT_BLOCK64) return 64;
         if (prm.variant == MD_VARIANT_BLOCK256) return 256;
         return kStepBlockMixed;

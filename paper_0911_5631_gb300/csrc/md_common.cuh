@@ -14,6 +14,9 @@ constexpr int kBlock = 256;
 // The final step of a call, which writes per-block energy partials, keeps
 // kBlock.
 constexpr int kStepBlockMixed = 128;
+// The same for the FP64 form: 128 threads, so that a block's warps share less
+// than 48 KB of shared memory (forces_fp64).
+constexpr int kStepBlockF64 = 128;
 // The step's closing work (counters, rebuild decision, next conditional
 // node) runs as a one-warp kernel after the step kernel rather than in the
 // step kernel's last block.
@@ -193,6 +196,14 @@ struct alignas(16) Args {
     float shell_inv;    // kShellBins / skin (0 without a skin)
     float shell_eps;    // rounding margin of the shell-bin bound (distance units)
     double close2;
+    // FP64 form: the payload of a pair coordinate is the position packed as
+    // three 21-bit fixed-point numbers, component d in units of M_d / 2^21
+    // modulo the period M_d = L_d / k_d, k_d whole, M_d >= 3 r_n, so that a
+    // difference is the nearest image's separation without a cell code.  It
+    // serves an FP32 distance test that no pair inside r_c fails.
+    unsigned long long pinc[3];  // cell width in units of M_d / 2^64: k_d 2^64 / G_d
+    float punit[3], pinv[3];     // M_d / 2^32 and 2^32 / M_d
+    float near2f;                // bound of the test: r_c^2 and the packing's rounding
 
     // per-atom state, storage order
     int* cell;          // cell index of the last binning

@@ -132,6 +132,10 @@ void fill_args_scalars(Args<P>& a, const md_plan_t& plan, const double box[3], i
         a.hwf_in[k] = (float)(0.5 * plan.w[k] * (1.0 - 1e-6));
         a.hw_in[k] = 0.5 * plan.w[k] * (1.0 - 1e-9);
         a.wf[k] = (float)plan.w[k];
+        const double periods = std::fmax(1.0, std::floor(box[k] / (3.0 * (rc + skin))));
+        a.pinc[k] = (unsigned long long)((((unsigned __int128)(uint64_t)periods) << 64) / (unsigned)plan.G[k]);
+        a.punit[k] = (float)std::ldexp(box[k] / periods, -32);
+        a.pinv[k] = (float)std::ldexp(periods / box[k], 32);
     }
     a.ntiles = (int)((plan.n_cells + kScanTile - 1) / kScanTile);
     a.nblocks = (int)((n + kBlock - 1) / kBlock);
@@ -157,6 +161,16 @@ void fill_args_scalars(Args<P>& a, const md_plan_t& plan, const double box[3], i
     a.ushiftf = (float)plan.ushift;
     a.thr2 = 0.25 * skin * skin;
     a.thr2f = (float)(a.thr2 * (1.0 - 1e-5));
+    {
+        // Packed separations (Args::near2f): two truncations to whole units,
+        // and up to a unit each of borrow and of the bits below the unit, put
+        // a component within 2 units of the exact one (2.1 with the FP32
+        // rounding of the offsets)
+        double m = 0.0;
+        for (int k = 0; k < 3; k++) m = std::fmax(m, (double)a.punit[k]);
+        const double delta = 2.1 * 2048.0 * m;
+        a.near2f = (float)((a.rc2 + 4.0 * rc * delta + 3.0 * delta * delta) * (1.0 + 2e-6));
+    }
     a.close2 = 0.08;
     a.close2f = 0.08f;
     // |f_d| = (f/r) |d_d| < (f/r) r_c for an interacting pair; 2000 leaves

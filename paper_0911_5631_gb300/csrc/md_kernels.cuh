@@ -235,12 +235,6 @@ __device__ __forceinline__ bool bin_coord(const Args<P>& a, int d, double x, int
     return true;
 }
 
-// Shift -d w of a neighbour whose 2-bit cell-offset code is k (d = k - 1).
-template <class T>
-__device__ __forceinline__ T code_shift(unsigned k, T w) {
-    return k == 0u ? w : (k == 2u ? -w : T(0));
-}
-
 // ---------------------------------------------------------------------------
 // Conversions on the FP32 and integer pipes.  They follow the IEEE 754
 // binary32/binary64 encodings with round-to-nearest-even; values below the
@@ -384,6 +378,42 @@ struct Fix2 {
     }
 };
 
+// 1 / a.  The seed (rcp.approx.ftz.f64, good to about 2^-20) is refined by
+// one third-order step of Householder's iteration for the reciprocal,
+// y (1 + e + e^2) with e = 1 - a y, whose error e^3 is below 2^-53: three
+// FP64 operations where the division takes about ten.  An infinite seed
+// (a = 0) is the result.
+__device__ __forceinline__ double reciprocal(double a) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-a, y, 1.0);
+    const double r = fma(y, fma(e, e, e), y);
+    return (__double2hiint(y) & 0x7fffffff) == 0x7ff00000 ? y : r;
+}
+
+// a < b for non-negative doubles (a NaN counts as large), compared as
+// integers: a comparison on the FP64 pipe costs as much as an addition.
+__device__ __forceinline__ bool less_bits(double a, double b) {
+    return __double_as_longlong(a) < __double_as_longlong(b);
+}
+
+// Payload of a pair coordinate.  FP64 form: the position packed for the FP32
+// distance test (Args::pinc), from the offsets p in the cell; mixed form:
+// unused.
+__device__ __forceinline__ long long pair_payload(const Args<F64>& a, int cell, double px, double py, double pz) {
+    const double p[3] = {px, py, pz};
+    unsigned long long w = 0;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const unsigned c = ((unsigned)cell >> (10 * d)) & 1023u;
+        const unsigned centre = (unsigned)((a.pinc[d] * (unsigned long long)c + (a.pinc[d] >> 1)) >> 32);
+        const unsigned u = centre + (unsigned)__float2int_rn(cvt::f32(p[d]) * a.pinv[d]);
+        w |= (unsigned long long)(u >> 11) << (21 * d);
+    }
+    return (long long)w;
+}
+__device__ __forceinline__ int pair_payload(const Args<Mixed>&, int, float, float, float) { return 0; }
+
 // Pair coordinate of one component from build offset and displacement.
 __device__ __forceinline__ float pair_coord(float pb, double o) { return pb + cvt::f32(o); }
 __device__ __forceinline__ double pair_coord(double pb, double o) { return __dadd_rn(pb, o); }
@@ -430,8 +460,8 @@ __device__ __forceinline__ double moved(double pb, double o, double& p) {
 __device__ __forceinline__ float4 make_pos4(float x, float y, float z, int j) {
     return make_float4(x, y, z, __int_as_float(j));
 }
-__device__ __forceinline__ double4_32a make_pos4(double x, double y, double z, int j) {
-    return make_double4_32a(x, y, z, __longlong_as_double((long long)j));
+__device__ __forceinline__ double4_32a make_pos4(double x, double y, double z, long long j) {
+    return make_double4_32a(x, y, z, __longlong_as_double(j));
 }
 __device__ __forceinline__ float4 ld_pos4(const float4* p) { return __ldg(p); }
 __device__ __forceinline__ double4_32a ld_pos4(const double4_32a* p) {
@@ -511,10 +541,10 @@ struct AccF64 {
     int close = 0;
     template <bool kEnergy>
     __device__ __forceinline__ void force(const Args<F64>& a, double dx, double dy, double dz, double r2) {
-        close |= (r2 < a.close2);
-        double ir2 = 1.0 / r2;
+        close |= less_bits(r2, a.close2);
+        double ir2 = reciprocal(r2);
         double ir6 = ir2 * ir2 * ir2;
-        double fr = 48.0 * ir6 * (ir6 - 0.5) * ir2;
+        double fr = fma(48.0, ir6, -24.0) * ir6 * ir2;
         fx += fr * dx;
         fy += fr * dy;
         fz += fr * dz;
@@ -541,95 +571,140 @@ template <class P> struct AccOf;
 template <> struct AccOf<Mixed> { using type = AccMixed; };
 template <> struct AccOf<F64> { using type = AccF64; };
 
-// Per-thread queue of interacting pairs (separation, r^2) in shared memory,
-// slot-major so that a warp's accesses are contiguous.
-template <class P> struct Queue;
-template <> struct Queue<Mixed> {
-    using item = float4;
-    static constexpr int kSlots = 6;
-    __device__ __forceinline__ static item make(float x, float y, float z, float r2) { return make_float4(x, y, z, r2); }
-};
-template <> struct Queue<F64> {
-    using item = double4_32a;
-    static constexpr int kSlots = 3;
-    __device__ __forceinline__ static item make(double x, double y, double z, double r2) {
-        return make_double4_32a(x, y, z, r2);
-    }
-};
-
-// Shift -d w for each 6-bit cell-offset code, built per block in shared
-// memory (entries whose code has a component 3 are unused).
-template <class P>
-__device__ __forceinline__ void fill_shift_table(const Args<P>& a, typename P::pos4* tbl) {
-    using real = typename P::real;
-    if (threadIdx.x < 64) {
-        unsigned c = threadIdx.x;
-        real w0, w1, w2;
-        if constexpr (P::kFp64) { w0 = a.w[0]; w1 = a.w[1]; w2 = a.w[2]; }
-        else { w0 = a.wf[0]; w1 = a.wf[1]; w2 = a.wf[2]; }
-        tbl[c] = make_pos4(code_shift<real>(c & 3u, w0), code_shift<real>((c >> 2) & 3u, w1),
-                           code_shift<real>((c >> 4) & 3u, w2), 0);
-    }
-}
-
-// Forces on atom i from its neighbour-list column (Sec. 3.4: W_{m,i}, m_i),
-// in two phases.  Phase 1 reads the entries (four at a time, so several
-// independent loads are in flight), tests r^2 < r_c^2 and queues the
-// interacting separations; phase 2 evaluates the pair term for the queued
-// pairs only.  A warp thus runs the expensive pair term as often as its
-// busiest atom has interacting partners instead of as often as it has
-// neighbour entries.  Pairs beyond the queue are evaluated at once.  The
-// first `staged` rows of the warp's column block are already in shared
-// memory (rows), the rest is read from global memory.
-template <class P, bool kEnergy>
-__device__ __forceinline__ void forces_from_list(const Args<P>& a, int cnt, const int* col, const int* rows, int staged,
-                                                 typename P::real qx, typename P::real qy, typename P::real qz,
-                                                 const typename P::pos4* __restrict__ pc,
-                                                 const typename P::pos4* __restrict__ shift,
-                                                 typename Queue<P>::item* queue,
-                                                 typename AccOf<P>::type& acc) {
-    using real = typename P::real;
-    using pos4 = typename P::pos4;
-    constexpr int kQ = Queue<P>::kSlots;
+// Forces on a warp's 32 atoms from their neighbour-list columns (Sec. 3.4:
+// W_{m,i}, m_i), FP64 form.
+//
+// What bounds the FP64 step is the FP64 pipe: two lanes per clock per SM, 16
+// clocks for a warp's instruction however many of its lanes are active.  So
+// the FP64 work is reduced to the interacting pairs and spread over full
+// warps.  First each lane tests its entries in FP32 on the packed positions
+// (8 bytes gathered per entry, no cell code: pair_payload) and keeps the
+// entries of the survivors in its column of the staged rows, in place.  Then
+// the warp's survivors, about 4.5 per atom, are numbered in lane order and
+// evaluated 32 at a time with the exact test, and every lane adds up its own
+// atom's terms, in list order.  A pair's FP64 operations are 3 for the
+// separation (the atom's coordinate seen from each of the three cells of a
+// direction is prepared once, in `tab`), 3 for r^2, 3 for the reciprocal, 5
+// for f/r, 3 for the force and 3 additions at the end.  Every lane testing
+// its entries in FP64 and evaluating its own queue took 470 us per step at
+// 1M atoms, most of a warp's lanes idle at each FP64 instruction; this takes
+// 250 us, with the FP64 pipe 82 % busy.
+//
+// rows: the warp's staged rows (kStageRows x 32 ints); tab: 9 x 32 doubles;
+// res: kRes x (3, or 5 with kEnergy) doubles.  Every lane of the warp must
+// call it (cnt = 0 for a lane without an atom).
+template <bool kEnergy, int kRes>
+__device__ __forceinline__ void forces_fp64(const Args<F64>& a, int cnt, const int* col, int* rows, int staged,
+                                            double qx, double qy, double qz, unsigned long long qw,
+                                            const double4_32a* __restrict__ pc, double* tab, double* res,
+                                            AccF64& acc) {
+    constexpr unsigned kFull = 0xffffffffu;
     const unsigned jmask = a.jmask;  // entries are always < n; the mask only guards memory
+    const int lane = threadIdx.x & 31;
+    // the coordinate as seen from a neighbour cell at offset d = k - 1: q - d w
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        tab[(0 + k) * 32 + lane] = k == 0 ? __dadd_rn(qx, a.w[0]) : (k == 1 ? qx : __dsub_rn(qx, a.w[0]));
+        tab[(3 + k) * 32 + lane] = k == 0 ? __dadd_rn(qy, a.w[1]) : (k == 1 ? qy : __dsub_rn(qy, a.w[1]));
+        tab[(6 + k) * 32 + lane] = k == 0 ? __dadd_rn(qz, a.w[2]) : (k == 1 ? qz : __dsub_rn(qz, a.w[2]));
+    }
     int nq = 0;
-    for (int m = 0; m < cnt; m += 4) {
+    auto flush = [&]() {
+        int incl = nq;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int excl = incl - nq, total = __shfl_sync(kFull, incl, 31);
+        __syncwarp();
+        for (int base = 0; base < total; base += kRes) {
+            const int top = min(total - base, kRes);
+            for (int r = 0; r < top; r += 32) {
+                const int p = base + r + lane;
+                int own = 0;  // lanes whose inclusive count is <= p: the item's owner
+#pragma unroll
+                for (int st = 16; st > 0; st >>= 1)
+                    if (__shfl_sync(kFull, incl, own + st - 1) <= p) own += st;
+                own = min(own, 31);
+                const int first = __shfl_sync(kFull, excl, own);
+                if (r + lane >= top) continue;
+                const unsigned e = (unsigned)rows[(p - first) * 32 + own];
+                const double2* pj = reinterpret_cast<const double2*>(pc + (e & jmask));
+                const double2 pxy = __ldg(pj);
+                const double pz = __ldg(reinterpret_cast<const double*>(pj + 1));
+                const unsigned c = e >> kCodeShift;
+                const double dx = tab[(c & 3u) * 32 + own] - pxy.x;
+                const double dy = tab[(3 + ((c >> 2) & 3u)) * 32 + own] - pxy.y;
+                const double dz = tab[(6 + (c >> 4)) * 32 + own] - pz;
+                const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+                double g[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+                if (less_bits(r2, a.rc2)) {
+                    acc.close |= less_bits(r2, a.close2);
+                    const double ir2 = reciprocal(r2);
+                    const double ir6 = ir2 * ir2 * ir2;
+                    const double fr = fma(48.0, ir6, -24.0) * ir6 * ir2;
+                    g[0] = fr * dx;
+                    g[1] = fr * dy;
+                    g[2] = fr * dz;
+                    if constexpr (kEnergy) {
+                        g[3] = fma(fma(4.0, ir6, -4.0), ir6, a.ushift);
+                        g[4] = fr * r2;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < (kEnergy ? 5 : 3); k++) res[k * kRes + r + lane] = g[k];
+            }
+            __syncwarp();
+            const int t1 = min(excl + nq - base, top);
+            for (int t = max(excl - base, 0); t < t1; t++) {
+                acc.fx += res[t];
+                acc.fy += res[kRes + t];
+                acc.fz += res[2 * kRes + t];
+                if constexpr (kEnergy) {
+                    acc.u += res[3 * kRes + t];
+                    acc.w += res[4 * kRes + t];
+                }
+            }
+            __syncwarp();
+        }
+        nq = 0;
+    };
+    const int cmax = __reduce_max_sync(kFull, cnt);
+    for (int m = 0; m < cmax; m += 4) {
         unsigned e[4];
-        pos4 pj[4];
+        unsigned long long w[4];
 #pragma unroll
         for (int k = 0; k < 4; k++)
-            e[k] = (m + k < cnt) ? (unsigned)(m + k < staged ? rows[(m + k) * 32 + (threadIdx.x & 31)]
-                                                             : __ldcs(col + (size_t)(m + k) * 32))
-                                 : 0u;
+            e[k] = m + k < cnt ? (unsigned)(m + k < staged ? rows[(m + k) * 32 + lane]
+                                                           : __ldcs(col + (size_t)(m + k) * 32))
+                               : 0u;
 #pragma unroll
         for (int k = 0; k < 4; k++)
-            if (m + k < cnt) pj[k] = ld_pos4(pc + (e[k] & jmask));
+            if (m + k < cnt)
+                w[k] = __ldg(reinterpret_cast<const unsigned long long*>(pc + (e[k] & jmask)) + 3);
 #pragma unroll
         for (int k = 0; k < 4; k++) {
             if (m + k < cnt) {
-                const pos4 sh = shift[e[k] >> kCodeShift];
-                real dx = (qx - pj[k].x) + sh.x;
-                real dy = (qy - pj[k].y) + sh.y;
-                real dz = (qz - pj[k].z) + sh.z;
-                real rr = acc.r2(dx, dy, dz);
-                if (acc.inside(a, rr)) {
-                    if (nq < kQ) queue[nq * blockDim.x + threadIdx.x] = Queue<P>::make(dx, dy, dz, rr);
-                    else acc.template force<kEnergy>(a, dx, dy, dz, rr);
+                const unsigned long long D = qw - w[k];
+                const unsigned lo = (unsigned)D, hi = (unsigned)(D >> 32);
+                const float ex = (float)(int)(lo << 11) * a.punit[0];
+                const float ey = (float)(int)__funnelshift_l(lo, hi, 22) * a.punit[1];
+                const float ez = (float)(int)(hi << 1) * a.punit[2];
+                if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) < a.near2f) {
+                    rows[nq * 32 + lane] = (int)e[k];  // (row nq has been read: nq <= m + k)
                     nq++;
                 }
             }
         }
+        if (__any_sync(kFull, nq > kStageRows - 4)) flush();
     }
-    const int nk = min(nq, kQ);
-    for (int k = 0; k < nk; k++) {
-        const auto d = queue[k * blockDim.x + threadIdx.x];
-        acc.template force<kEnergy>(a, d.x, d.y, d.z, d.w);
-    }
+    if (__any_sync(kFull, nq > 0)) flush();
 }
 
-// Mixed-form counterpart of forces_from_list, in one pass: each entry's
-// pair term is evaluated as soon as its distance test passes.  Here the
-// shared-memory queue and the shift table cost more L1 data-pipe
+// Mixed-form counterpart of forces_fp64, in one pass: each entry's pair
+// term is evaluated as soon as its distance test passes.  Here a
+// shared-memory queue and a shift table cost more L1 data-pipe
 // wavefronts than the divergence they save, so the shift
 // -d w = (1 - k) w of each component (k the 2-bit code) is computed from
 // the code, and the staged rows and the rest of the column run as two loops
@@ -788,7 +863,8 @@ __device__ __forceinline__ void set_state_item(const Args<P>& a, int64_t i) {
         a.vy[i] = cvt::f32(a.io_vel[3 * i + 1]);
         a.vz[i] = cvt::f32(a.io_vel[3 * i + 2]);
     }
-    a.pA[i] = make_pos4(pair_coord(pb[0], o[0]), pair_coord(pb[1], o[1]), pair_coord(pb[2], o[2]), 0);
+    const real p0 = pair_coord(pb[0], o[0]), p1 = pair_coord(pb[1], o[1]), p2 = pair_coord(pb[2], o[2]);
+    a.pA[i] = make_pos4(p0, p1, p2, pair_payload(a, a.cell[i], p0, p1, p2));
 }
 
 template <class P>
@@ -869,7 +945,8 @@ __device__ __forceinline__ int bin_item(const Args<P>& a, int64_t i) {
     if (bad) atomicOr(&C->error, kErrUnstable);
     a.cell[i] = pack_cell(cc[0], cc[1], cc[2]);
     typename P::pos4* pc = C->parity ? a.pB : a.pA;
-    pc[i] = make_pos4(pair_coord(pb[0], o[0]), pair_coord(pb[1], o[1]), pair_coord(pb[2], o[2]), 0);
+    const real p0 = pair_coord(pb[0], o[0]), p1 = pair_coord(pb[1], o[1]), p2 = pair_coord(pb[2], o[2]);
+    pc[i] = make_pos4(p0, p1, p2, pair_payload(a, pack_cell(cc[0], cc[1], cc[2]), p0, p1, p2));
     const int c = cell_index(cc[0], cc[1], cc[2], a.G);
     a.rank[i] = atomicAdd(&a.count[c], 1);
     return c;
@@ -1050,7 +1127,8 @@ __device__ __forceinline__ void commit_item(const Args<P>& a, int64_t s) {
     a.ox[s] = ox; a.oy[s] = oy; a.oz[s] = oz;
     a.vx[s] = a.s_vx[s]; a.vy[s] = a.s_vy[s]; a.vz[s] = a.s_vz[s];
     typename P::pos4* pc = C->parity ? a.pB : a.pA;
-    pc[s] = make_pos4(pair_coord(pbx, ox), pair_coord(pby, oy), pair_coord(pbz, oz), 0);
+    const auto p0 = pair_coord(pbx, ox), p1 = pair_coord(pby, oy), p2 = pair_coord(pbz, oz);
+    pc[s] = make_pos4(p0, p1, p2, pair_payload(a, a.s_cell[s], p0, p1, p2));
 }
 
 template <class P>
@@ -1692,7 +1770,7 @@ __device__ __forceinline__ bool kickdrift_item(const Args<P>& a, int64_t i, type
     real d2 = moved(a.pbx[i], ox, px) + moved(a.pby[i], oy, py) + moved(a.pbz[i], oz, pz);
     a.vx[i] = vx; a.vy[i] = vy; a.vz[i] = vz;
     a.ox[i] = ox; a.oy[i] = oy; a.oz[i] = oz;
-    pc[i] = make_pos4(px, py, pz, 0);
+    pc[i] = make_pos4(px, py, pz, pair_payload(a, P::kFp64 ? a.cell[i] : 0, px, py, pz));
     d2b = d2_bits(d2);
     if constexpr (P::kFp64) return d2 >= a.thr2;
     else return d2 >= a.thr2f;
@@ -1768,6 +1846,11 @@ __device__ __forceinline__ void stage_wait() {
     }
 }
 
+// Terms a warp of the FP64 list form holds at a time: the warp's survivors of
+// most fluids in the plain step; one round in the final step, whose five sums
+// and 256-thread blocks leave less shared memory.
+__host__ __device__ constexpr int f64_results(bool final_step) { return final_step ? 32 : 160; }
+
 // The per-atom part of a step (Sec. 3.1 (c)-(e) and (a) of the next step):
 // forces of atom i, then either the final-step work (v_n, stored forces,
 // KE/PE/W terms) or the next half kick, the drift into the other pair
@@ -1775,28 +1858,33 @@ __device__ __forceinline__ void stage_wait() {
 // per-replica engine.
 template <class P, bool kCells, bool kFinal, bool kLdg = true, bool kRows = false, bool kHwCvt = false>
 __device__ __forceinline__ void step_atom(const Args<P>& a, int64_t i, bool in, bool active, bool init, bool energy,
-                                          int cnt, const int* col, const int* rows, int staged,
+                                          int cnt, const int* col, int* rows, int staged,
                                           const typename P::pos4* __restrict__ pc, typename P::pos4* pn,
-                                          const typename P::pos4* s_shift, typename Queue<P>::item* s_queue,
-                                          bool& far, bool& close, double& ke, double& pe, double& vir,
+                                          double* f64_tab, double* f64_res, bool& far, bool& close, double& ke, double& pe, double& vir,
                                           unsigned& d2b) {
     using real = typename P::real;
     using vel = typename P::vel;
     using pos4 = typename P::pos4;
-    if (!(active && in)) return;
+    // (the FP64 list form's lanes work together: lanes without an atom take part)
+    constexpr bool kTogether = P::kFp64 && !kCells;
+    if (!active || !(in || kTogether)) return;
     {
-        const pos4 qi = ld_pos4(pc + i);
+        const pos4 qi = ld_pos4(pc + (in ? i : 0));
         const real qx = qi.x, qy = qi.y, qz = qi.z;
         typename AccOf<P>::type acc;
-        if (kFinal && energy) {
+        if constexpr (kTogether) {
+            forces_fp64<kFinal, f64_results(kFinal)>(a, in ? cnt : 0, col, rows, staged, qx, qy, qz,
+                                                     (unsigned long long)__double_as_longlong(qi.w), pc, f64_tab,
+                                                     f64_res, acc);
+            if (!in) {
+                close = acc.close != 0;
+                return;
+            }
+        } else if (kFinal && energy) {
             if constexpr (kCells) forces_from_cells<P, kFinal>(a, (int)i, qx, qy, qz, pc, acc);
-            else if constexpr (P::kFp64)
-                forces_from_list<P, kFinal>(a, cnt, col, rows, staged, qx, qy, qz, pc, s_shift, s_queue, acc);
             else forces_mixed<kFinal, kLdg, kRows>(a, cnt, col, rows, staged, qx, qy, qz, pc, acc);
         } else {
             if constexpr (kCells) forces_from_cells<P, false>(a, (int)i, qx, qy, qz, pc, acc);
-            else if constexpr (P::kFp64)
-                forces_from_list<P, false>(a, cnt, col, rows, staged, qx, qy, qz, pc, s_shift, s_queue, acc);
             else forces_mixed<false, kLdg, kRows>(a, cnt, col, rows, staged, qx, qy, qz, pc, acc);
         }
         close = acc.close != 0;
@@ -1829,7 +1917,7 @@ __device__ __forceinline__ void step_atom(const Args<P>& a, int64_t i, bool in, 
             real d2 = moved<kHwCvt>(pbx, ox, px) + moved<kHwCvt>(pby, oy, py) + moved<kHwCvt>(pbz, oz, pz);
             a.vx[i] = vx; a.vy[i] = vy; a.vz[i] = vz;
             a.ox[i] = ox; a.oy[i] = oy; a.oz[i] = oz;
-            pn[i] = make_pos4(px, py, pz, 0);
+            pn[i] = make_pos4(px, py, pz, pair_payload(a, P::kFp64 && !kCells ? a.cell[i] : 0, px, py, pz));
             d2b = d2_bits(d2);
             if constexpr (P::kFp64) far = d2 >= a.thr2;
             else far = d2 >= a.thr2f;
@@ -1884,20 +1972,19 @@ __device__ __forceinline__ void close_step(const Args<P>& a, const CloseIn& in, 
 // variant with kB != kBlock serves the plain steps only: the final step,
 // which writes per-block energy partials, always runs with kBlock.
 template <class P, bool kCells, bool kFinal, int kB = kBlock, bool kLdg = true, bool kRows = false>
-__global__ void __launch_bounds__(kB, P::kFp64 ? 3 : 5 * kBlock / kB) k_step(Args<P> a, int mode,
-                                                                             cudaGraphConditionalHandle next,
-                                                                             int has_next) {
+__global__ void __launch_bounds__(kB, P::kFp64 ? (kB == kBlock ? 3 : 5) : 5 * kBlock / kB)
+    k_step(Args<P> a, int mode, cudaGraphConditionalHandle next, int has_next) {
     static_assert(!kFinal || kB == kBlock, "the final step runs with kBlock threads");
     using real = typename P::real;
     using vel = typename P::vel;
     using pos4 = typename P::pos4;
     __shared__ double shs[kB / 32];
-    constexpr bool kTable = P::kFp64 && !kCells;  // shift table and pair queue (FP64 list form)
-    __shared__ pos4 s_shift[kTable ? 64 : 1];
-    __shared__ typename Queue<P>::item s_queue[kTable ? Queue<P>::kSlots * kB : 1];
+    constexpr bool kTable = P::kFp64 && !kCells;  // per-warp tables of the FP64 list form
+    constexpr int kRes = f64_results(kFinal) * (kFinal ? 5 : 3);
+    __shared__ double s_tab[kTable ? 9 * kB : 1];
+    __shared__ double s_res[kTable ? kRes * (kB / 32) : 1];
     __shared__ __align__(16) int s_rows[(kCells || kRows) ? 4 : kStageRows * kB];
     Counters* C = a.ctr;
-    if constexpr (kTable) fill_shift_table<P>(a, s_shift);
     // Requests that do not depend on the counters go out first, so their
     // latency overlaps the counter read: the first rows of the warp's
     // neighbour column block (copied to shared memory; rows below the
@@ -1912,8 +1999,7 @@ __global__ void __launch_bounds__(kB, P::kFp64 ? 3 : 5 * kBlock / kB) k_step(Arg
     int* rows = s_rows + (threadIdx.x >> 5) * (kStageRows * 32);
     stage_rows<P, kCells, kRows>(a, i, C->reach, rows, cnt, staged, col);
     stage_wait<kCells || kRows>();
-    // the FP64 list form's block barrier also orders the table fill before its use
-    const View vw = (kTable || !kStepTailNode || !kWarpView) ? load_view(C) : load_view_warp(C);
+    const View vw = (!kStepTailNode || !kWarpView) ? load_view(C) : load_view_warp(C);
     const int err = vw.err;
     const long long left = vw.left;
     const int par = vw.par;
@@ -1931,7 +2017,9 @@ __global__ void __launch_bounds__(kB, P::kFp64 ? 3 : 5 * kBlock / kB) k_step(Arg
     double ke = 0.0, pe = 0.0, vir = 0.0;
     unsigned d2b = 0u;
     step_atom<P, kCells, kFinal, kLdg, kRows, true>(a, i, in, active, init, energy, cnt, col, rows, staged, pc, pn,
-                                                    s_shift, s_queue, far, close, ke, pe, vir, d2b);
+                                                    s_tab + (kTable ? (threadIdx.x >> 5) * (9 * 32) : 0),
+                                                    s_res + (kTable ? (threadIdx.x >> 5) * kRes : 0), far, close, ke,
+                                                    pe, vir, d2b);
     if (__any_sync(0xffffffffu, far) && (threadIdx.x & 31) == 0) atomicOr(&C->far_flag, 1u);
     if (__any_sync(0xffffffffu, close) && (threadIdx.x & 31) == 0) atomicOr(&C->close_flag, 1);
     warp_max_into(d2b, d2_word(a));  // the running maximum of the squared displacement
@@ -2566,7 +2654,7 @@ KernelTable<P> make_kernel_table() {
     t.kickdrift = (void*)k_kickdrift<P>;
     t.step_tail = (void*)k_step_tail<P, false>;
     t.step_tail_final = (void*)k_step_tail<P, true>;
-    if constexpr (P::kFp64) t.step_list = (void*)k_step<P, false, false>;
+    if constexpr (P::kFp64) t.step_list = (void*)k_step<P, false, false, kStepBlockF64>;
     else t.step_list = (void*)k_step<P, false, false, kStepBlockMixed>;
     t.step_list_final = (void*)k_step<P, false, true>;
     t.step_cells = (void*)k_step<P, true, false>;

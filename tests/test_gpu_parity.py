@@ -241,6 +241,34 @@ def test_newton_third_law_in_result(prec):
     s.close()
 
 
+# sizes around a warp of 32 atoms and a block of 128, a density whose atoms
+# have more interacting pairs than a warp holds entries or results for (one
+# round of evaluation is not enough), a box that is no cube
+@pytest.mark.parametrize("n,rho,jit,aspect", [(31, 0.35, 0.2, (1, 1, 1)), (33, 0.35, 0.2, (1, 1, 1)),
+                                              (129, 0.8, 0.1, (1, 1, 1)), (700, 2.5, 0.02, (1, 1, 1)),
+                                              (1025, 1.8, 0.03, (1.2, 0.9, 1.0))])
+def test_fp64_forces_at_the_edges_of_the_warp_evaluation(n, rho, jit, aspect):
+    pos, vel, L = state(n, rho, 1.0, 41, jitter=jit, aspect=aspect)
+    s = sim(pos, vel, L, skin=0.3, precision="fp64")
+    pw = oracle.wrap(pos, L)
+    f_ref, U, W = oracle.forces_cells(pw, L, oracle_grid(L, RC), RC, 1.0)
+    assert rel_rms(s.forces(), f_ref) <= FORCE_TOL["fp64"]
+    m = s.measure()
+    assert m["pe"] == pytest.approx(U, rel=10 * FORCE_TOL["fp64"])
+    assert m["virial"] == pytest.approx(W, rel=10 * FORCE_TOL["fp64"])
+    # the plain step's kernel, one step and the next (which uses its forces)
+    ref = oracle.run(pw, vel, L, RC, 0.3, 1e-4, 2)
+    s2 = md.Simulation(L, n, RC, 0.3, 1e-4, precision="fp64")
+    s2.set_state(pos, vel)
+    s2.step(2)
+    p, v = s2.get_state()
+    # two steps' impulses, to the force tolerance of each
+    f_rms = float(np.sqrt(np.mean(f_ref ** 2)))
+    assert np.sqrt(np.mean((v - ref["vel"]) ** 2)) <= 2e-4 * f_rms * 10 * FORCE_TOL["fp64"] + 1e-14
+    s.close()
+    s2.close()
+
+
 _trajectory_tol = trajectory_tol
 
 
