@@ -12,6 +12,7 @@
 // reads the rebuild flag before each step.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -113,6 +114,8 @@ struct Sim : SimBase {
 
     bool profiling = false;
     std::vector<cudaEvent_t> ev;
+    unsigned long long* run_words = nullptr;  // grid barrier of the one-launch step loop
+    int run_blocks_max = -1;  // blocks of it that fit the device at once (-1: not yet asked)
     int64_t launches = 0;
     int64_t graph_launches = 0;
     int64_t steps_run = 0;
@@ -202,6 +205,7 @@ struct Sim : SimBase {
         chk(alloc(&a.part, (size_t)3 * a.nblocks));
         chk(alloc(&a.ctr, 1));
         chk(alloc(&a.d2b, (size_t)kD2Buckets * 32));
+        chk(alloc(&run_words, (size_t)4 * kRunWordStride));
         chk(alloc(&a.io_pos, (size_t)3 * n)); chk(alloc(&a.io_vel, (size_t)3 * n));
         if (r) return r;
         r = alloc_nbr(a.cap);
@@ -371,8 +375,10 @@ struct Sim : SimBase {
 
     // K steps, plain ones or (final_node, K = 1) the one that may be a call's
     // last: k_cond, then per step the step kernel and its closing kernel,
-    // with a conditional rebuild node before every m-th step (every step in
-    // the cell-list-only form, which rebuilds at each).  The closing kernel
+    // with a conditional rebuild node before every m-th step.  The
+    // cell-list-only form rebuilds at every step: its graphs hold the
+    // rebuild's kernels themselves (a conditional node costs about 5 us), each
+    // of which returns at once should the device flag not be set.  The closing kernel
     // before a conditional node sets its handle; a step after another whose
     // rebuild is due waits for the next conditional node.
     int build_chunk(Chunk& c, int K, bool final_node) {
@@ -432,6 +438,47 @@ struct Sim : SimBase {
 
     int graph_kernels_per_step() const { return 1; }
 
+    // Whether plain steps run in the one-launch loop of md_run.cuh: the mixed
+    // form with sorted lists and the default kernels, and a system whose
+    // blocks are all resident at once (up to 29184 atoms).  It wins wherever
+    // it applies: 100 steps and their read-back take 0.66 ms instead of 1.77
+    // at 2048 atoms and 1.15 ms instead of 2.05 at 20011.
+    bool use_run() {
+        if (P::kFp64 || prm.cell_list_only || !prm.shell_bins || prm.variant != 0 || warp_build() ||
+            use_direct_build(box, a.n, plan.rn))
+            return false;
+        const int block = run_block(a.n);
+        if (block == 0) return false;
+        if (run_blocks_max < 0) {
+            int coop = 0, sms = 0, per_sm = 0;
+            run_blocks_max = 0;
+            if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess || !coop ||
+                cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, run_fn(block), block, 0) != cudaSuccess) {
+                cudaGetLastError();
+                return false;
+            }
+            run_blocks_max = std::min(per_sm * sms, kRunMaxBlocks);
+        }
+        return run_grid(block) <= run_blocks_max;
+    }
+    void* run_fn(int block) const { return block == 128 ? kt.run_small : kt.run; }
+    int run_grid(int block) const { return (int)((a.n * kRunLanes + block - 1) / block); }
+
+    // Queues `count` plain steps as one-launch loops.
+    int run_loop(int64_t count) {
+        const int block = run_block(a.n);
+        while (count > 0) {
+            long long k = std::min<int64_t>(count, kRunSteps);
+            void* p[] = {(void*)&a, (void*)&k, (void*)&run_words};
+            MD_CUDA(cudaMemsetAsync(run_words, 0, sizeof(unsigned long long) * 4 * kRunWordStride, stream));
+            MD_CUDA(cudaLaunchCooperativeKernel(run_fn(block), dim3(run_grid(block)), dim3(block), p, 0, stream));
+            launches++;
+            count -= k;
+        }
+        return MD_OK;
+    }
+
     // Enqueues nsteps (rebuild?, force + integrate) pairs.
     int run_steps(int64_t nsteps) {
         if (nsteps <= 0) return MD_OK;
@@ -439,6 +486,11 @@ struct Sim : SimBase {
             // (a plain step must not meet a call's last one: steps that wait
             // for a rebuild only leave more to run, never fewer)
             int64_t left = nsteps - 1;
+            if (left > 0 && use_run()) {
+                int r = run_loop(left);
+                if (r) return r;
+                left = 0;
+            }
             for (int k = 0; k < kNumChunks; k++) {
                 int r = replay(plain[k], kChunks[k], false, left / kChunks[k]);
                 if (r) return r;
@@ -823,7 +875,7 @@ struct Sim : SimBase {
         std::memset(out, 0, sizeof(*out));
         // every rebuild branch that ran launched its kernels
         int per_rebuild = prm.cell_list_only ? 7 : 8;
-        int64_t body = prm.use_graphs && !profiling ? (int64_t)c.rebuilds * per_rebuild : 0;
+        int64_t body = prm.use_graphs && !profiling ? (int64_t)(c.rebuilds - c.run_rebuilds) * per_rebuild : 0;
         out->launches = launches + body;
         out->step_kernel_launches = step_launches;
         out->step_kernel_ms = step_ms;

@@ -73,6 +73,20 @@ constexpr int kD2Buckets = 64;
 constexpr int kEnsBuildStage = 16;
 static_assert(kEnsBuildStage < 256, "one byte per shell bin in a 64-bit word");
 constexpr int kEnsSmemInts = kStageRows > 2 * kEnsBuildStage ? kStageRows : 2 * kEnsBuildStage;
+// Lanes that share an atom in the force kernel of the cell-list-only variant.
+constexpr int kCellLanes = 8;
+// The one-launch step loop of small systems (md_run.cuh): kRunLanes lanes per
+// atom; blocks of 128, 256 or 384 threads, two of the largest on an SM (with
+// 80 registers a thread), so that every block of the launch is resident;
+// kRunMaxBlocks blocks at most.
+constexpr int kRunLanes = 4;
+constexpr int kRunMaxBlock = 384;
+constexpr int kRunMaxBlocks = 304;
+// Steps of one such launch at most (some milliseconds), and polls of a word
+// before a wait is given up (at half a microsecond or more each).
+constexpr int kRunSteps = 2048;
+constexpr int kRunPolls = 1 << 21;
+constexpr int kRunWordStride = 16;  // 64-bit words between the barrier's four words
 // Elements per block of the cell-count scan (kBlock threads x 8).
 constexpr int kScanTile = 2048;
 // Largest neighbour capacity of the mixed form (its fixed-point partial
@@ -126,6 +140,7 @@ struct Counters {
     long long reorders;        // reorders since the state was loaded
     long long list_entries;    // neighbour-list length at the last build
     long long list_reads;      // entries the profiled steps read (k_count_reads)
+    long long run_rebuilds;    // those of `rebuilds` done inside the one-launch step loop
     // reduced measurement of the last finalize
     double ke, pe, virial;
 };

@@ -92,7 +92,7 @@ inline int resolve_plan(const double box[3], int64_t n, double rc, double skin, 
     int64_t ncol = (n + 31) / 32 * 32;
     out->device_bytes = per_atom * n + 2 * pos4_b * (pair_slots(n) - n) /*pair buffers padded*/ + ncol * cap * 4 +
                         (2 * nc + 1) * 4 + ((nc + kScanTile - 1) / kScanTile) * 4 + 3 * nb * 8 +
-                        (int64_t)sizeof(Counters) + kD2Buckets * 32 * 4;
+                        (int64_t)sizeof(Counters) + kD2Buckets * 32 * 4 + 4 * kRunWordStride * 8;
     return MD_OK;
 }
 
@@ -111,6 +111,15 @@ inline bool use_warp_build(const md_params& p) { return p.build_kernel == MD_BUI
 inline bool use_direct_build(const double box[3], int64_t n, double rn) {
     const double nbar = 4.0 / 3.0 * M_PI * rn * rn * rn * (double)n / (box[0] * box[1] * box[2]);
     return nbar > kBuildStage;
+}
+
+// Threads per block of the one-launch step loop (md_run.cuh) for n atoms:
+// the smallest blocks that leave at most one on an SM (152), then the
+// largest, two on an SM.  0: too many atoms.
+inline int run_block(int64_t n) {
+    for (int b = 128; b <= kRunMaxBlock; b += 128)
+        if (n * kRunLanes <= (int64_t)b * 152) return b;
+    return n * kRunLanes <= (int64_t)kRunMaxBlock * kRunMaxBlocks ? kRunMaxBlock : 0;
 }
 
 // Scalar members of Args from a plan.

@@ -907,7 +907,7 @@ __global__ void k_clear_overflow(Counters* C) {
 // operation on the cell coordinate).  Refreshes the pair coordinate and
 // counts the atoms of each cell.
 template <class P>
-__device__ __forceinline__ int bin_item(const Args<P>& a, int64_t i) {
+__device__ __forceinline__ int bin_item(const Args<P>& a, int64_t i, int parity) {
     using real = typename P::real;
     Counters* C = a.ctr;
     int cc[3];
@@ -944,7 +944,7 @@ __device__ __forceinline__ int bin_item(const Args<P>& a, int64_t i) {
     }
     if (bad) atomicOr(&C->error, kErrUnstable);
     a.cell[i] = pack_cell(cc[0], cc[1], cc[2]);
-    typename P::pos4* pc = C->parity ? a.pB : a.pA;
+    typename P::pos4* pc = parity ? a.pB : a.pA;
     const real p0 = pair_coord(pb[0], o[0]), p1 = pair_coord(pb[1], o[1]), p2 = pair_coord(pb[2], o[2]);
     pc[i] = make_pos4(p0, p1, p2, pair_payload(a, pack_cell(cc[0], cc[1], cc[2]), p0, p1, p2));
     const int c = cell_index(cc[0], cc[1], cc[2], a.G);
@@ -966,7 +966,7 @@ __global__ void __launch_bounds__(kBlock) k_bin(Args<P> a, int guard) {
         C->list_entries = 0;
     }
     const int64_t i = gtid();
-    const int tile = i < a.n ? bin_item<P>(a, i) / kScanTile : -1;
+    const int tile = i < a.n ? bin_item<P>(a, i, C->parity) / kScanTile : -1;
     const unsigned peers = __match_any_sync(0xffffffffu, tile);
     if (tile >= 0 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&a.tile_sum[tile], __popc(peers));
 }
@@ -1022,10 +1022,14 @@ __global__ void __launch_bounds__(kBlock) k_scan_apply(Args<P> a, int guard) {
 // Places each atom at cell_start[cell] + rank (the cell's arrival order)
 // and clears the counts for the next binning.
 template <class P>
-__device__ __forceinline__ void scatter_item(const Args<P>& a, int64_t t) {
-    int slot = a.cell_start[cell_index_of_packed(a.cell[t], a.G)] + a.rank[t];
-    if (slot >= 0 && slot < a.n) a.order[slot] = (int)t;
-    else atomicOr(&a.ctr->error, kErrUnstable);
+__device__ __forceinline__ int scatter_item(const Args<P>& a, int64_t t) {
+    const int slot = a.cell_start[cell_index_of_packed(a.cell[t], a.G)] + a.rank[t];
+    if (slot >= 0 && slot < a.n) {
+        a.order[slot] = (int)t;
+        return slot;
+    }
+    atomicOr(&a.ctr->error, kErrUnstable);
+    return -1;
 }
 
 template <class P>
@@ -1086,10 +1090,8 @@ __global__ void __launch_bounds__(kBlock) k_cellsort(Args<P> a, int guard) {
 // Writes the cell-ordered FP32 coordinate copy used by the neighbour search
 // and, when a reorder is due, the state permuted into cell order (Sec. 3.5).
 template <class P>
-__device__ __forceinline__ void gather_item(const Args<P>& a, int64_t s) {
+__device__ __forceinline__ void gather_item(const Args<P>& a, int64_t s, int reorder) {
     using real = typename P::real;
-    Counters* C = a.ctr;
-    const int reorder = C->reorder_now;
     int i = a.order[s];
     real pbx = a.pbx[i], pby = a.pby[i], pbz = a.pbz[i];
     double ox = a.ox[i], oy = a.oy[i], oz = a.oz[i];
@@ -1111,14 +1113,13 @@ __global__ void __launch_bounds__(kBlock) k_gather(Args<P> a, int guard) {
     if (guard && !C->rebuild_flag) return;
     int64_t s = gtid();
     if (s >= a.n) return;
-    gather_item<P>(a, s);
+    gather_item<P>(a, s, C->reorder_now);
 }
 
 // Copies the permuted state back and rewrites the current pair buffer in
 // the new order (only when a reorder is due).
 template <class P>
-__device__ __forceinline__ void commit_item(const Args<P>& a, int64_t s) {
-    Counters* C = a.ctr;
+__device__ __forceinline__ void commit_item(const Args<P>& a, int64_t s, int parity) {
     a.cell[s] = a.s_cell[s];
     a.perm[s] = a.s_perm[s];
     auto pbx = a.s_pbx[s], pby = a.s_pby[s], pbz = a.s_pbz[s];
@@ -1126,7 +1127,7 @@ __device__ __forceinline__ void commit_item(const Args<P>& a, int64_t s) {
     a.pbx[s] = pbx; a.pby[s] = pby; a.pbz[s] = pbz;
     a.ox[s] = ox; a.oy[s] = oy; a.oz[s] = oz;
     a.vx[s] = a.s_vx[s]; a.vy[s] = a.s_vy[s]; a.vz[s] = a.s_vz[s];
-    typename P::pos4* pc = C->parity ? a.pB : a.pA;
+    typename P::pos4* pc = parity ? a.pB : a.pA;
     const auto p0 = pair_coord(pbx, ox), p1 = pair_coord(pby, oy), p2 = pair_coord(pbz, oz);
     pc[s] = make_pos4(p0, p1, p2, pair_payload(a, a.s_cell[s], p0, p1, p2));
 }
@@ -1138,7 +1139,7 @@ __global__ void __launch_bounds__(kBlock) k_commit(Args<P> a, int guard) {
     if (!C->reorder_now) return;
     int64_t s = gtid();
     if (s >= a.n) return;
-    commit_item<P>(a, s);
+    commit_item<P>(a, s, C->parity);
 }
 
 // Exact FP64 neighbour criterion r^2 < r_n^2 for atom i and atom j, whose
@@ -1236,7 +1237,7 @@ __device__ __noinline__ int build_all(const Args<P>& a, int64_t s) {
         const unsigned code = (unsigned)((dx + 1) | ((dy + 1) << 2) | ((dz + 1) << 4));
         for (int t = a.cell_start[c]; t < end; t++) {
             if (t == (int)s) continue;
-            const float4 pj = __ldg(a.cand + t);
+            const float4 pj = a.cand[t];  // (written by the same kernel in the persistent engines)
             const float ex = (ci.x - (float)dx * a.wf[0]) - pj.x;
             const float ey = (ci.y - (float)dy * a.wf[1]) - pj.y;
             const float ez = (ci.z - (float)dz * a.wf[2]) - pj.z;
@@ -2370,7 +2371,7 @@ template <class P>
 __device__ __noinline__ void ens_rebuild(const Args<P>& a, EnsShared& sh, int* stage, Team tm) {
     Counters* C = a.ctr;
     const int64_t n = a.n, t0 = tm.first(), dt = tm.stride();
-    for (int64_t i = t0; i < n; i += dt) bin_item<P>(a, i);
+    for (int64_t i = t0; i < n; i += dt) bin_item<P>(a, i, C->parity);
     tm.sync();
     if (tm.lead_block()) ens_scan<P>(a, sh);
     tm.sync();
@@ -2379,10 +2380,10 @@ __device__ __noinline__ void ens_rebuild(const Args<P>& a, EnsShared& sh, int* s
     tm.sync();
     for (int64_t c = t0; c < a.ncells; c += dt) cellsort_item<P>(a, c);
     tm.sync();
-    for (int64_t s = t0; s < n; s += dt) gather_item<P>(a, s);
+    for (int64_t s = t0; s < n; s += dt) gather_item<P>(a, s, C->reorder_now);
     tm.sync();
     if (C->reorder_now) {
-        for (int64_t s = t0; s < n; s += dt) commit_item<P>(a, s);
+        for (int64_t s = t0; s < n; s += dt) commit_item<P>(a, s, C->parity);
         tm.sync();
     }
     int mx = 0;
@@ -2631,6 +2632,12 @@ __global__ void __launch_bounds__(1024, 1) k_ensemble(const Args<P>* __restrict_
     }
 }
 
+}  // namespace md
+
+#include "md_run.cuh"
+
+namespace md {
+
 // ---------------------------------------------------------------------------
 // kernel table used by the host runtime (graph nodes and eager launches)
 // ---------------------------------------------------------------------------
@@ -2671,6 +2678,8 @@ KernelTable<P> make_kernel_table() {
     t.spin = (void*)k_spin<P>;
     if constexpr (!P::kFp64) {
         t.ensemble = (void*)k_ensemble<P>;
+        t.run_small = (void*)k_run<P, 128>;
+        t.run = (void*)k_run<P, kRunMaxBlock>;
         // ablation variants of the mixed list form: {plain, final}
         t.step_var[0][0] = (void*)k_step<P, false, false, kStepBlockMixed, false, false>;  // plain loads
         t.step_var[0][1] = (void*)k_step<P, false, true, kBlock, false, false>;
@@ -2682,6 +2691,7 @@ KernelTable<P> make_kernel_table() {
         t.step_var[3][1] = (void*)k_step<P, false, true, kBlock, true, false>;
     } else {
         t.ensemble = nullptr;
+        t.run_small = t.run = nullptr;
         for (auto& v : t.step_var) v[0] = v[1] = nullptr;
     }
     return t;

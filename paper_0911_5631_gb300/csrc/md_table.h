@@ -38,6 +38,8 @@ struct KernelTable {
     void* count_reads;
     void* spin;
     void* ensemble;  // mixed form only (nullptr for FP64)
+    void* run_small;  // the one-launch step loop of small systems, blocks of 128 threads
+    void* run;       // the one-launch step loop of small systems, mixed form only
     // step-kernel variants of the paper's ablations, mixed list form only
     // ({plain step, final step}; index = the MD_VARIANT_* bit position)
     void* step_var[4][2];

@@ -1,0 +1,67 @@
+"""The one-launch step loop of small systems against stream launches of the
+grid kernels, which share its arithmetic: positions and velocities are the
+same bits, and the counters the same numbers."""
+import numpy as np
+import pytest
+
+import paper_0911_5631_gb300 as md
+from mdcheck import DT, RC, ensure_built, state
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    ensure_built()
+
+
+def _run(pos, vel, L, steps, skin, **kw):
+    s = md.Simulation(L, pos.shape[0], RC, skin, DT, **kw)
+    s.set_state(pos, vel)
+    for k in steps:
+        s.step(k)
+    out = s.get_state() + (s.measure(), s.cells(), s.neighbor_pairs()[1])
+    s.close()
+    return out
+
+
+# sizes around a block's atoms (32, 64, 128), the changes of block size (a
+# block per SM of 152) and the largest system of the loop; hot states with a
+# thin skin that rebuild every few steps, reorders at almost every rebuild;
+# a state whose lists are longer than the lanes' registers and stages hold
+@pytest.mark.parametrize("n,rho,T,skin,reorder", [
+    (110, 0.8, 1.0, 0.3, 100), (129, 0.8, 2.0, 0.2, 3), (2048, 0.8, 1.0, 0.4, 100), (4864, 0.7, 2.0, 0.25, 10),
+    (4865, 0.7, 1.0, 0.4, 0), (9729, 0.9, 1.5, 0.4, 20), (20011, 0.6, 1.0, 0.5, 100), (29184, 0.8, 1.0, 0.4, 25),
+    (29185, 0.8, 1.0, 0.4, 25), (1500, 1.05, 2.0, 0.46, 30)])
+def test_run_loop_matches_stream_launches(n, rho, T, skin, reorder):
+    pos, vel, L = state(n, rho, T, 51, jitter=0.05)
+    steps = [1, 2, 60, 33]
+    a = _run(pos, vel, L, steps, skin, reorder_interval=reorder)
+    b = _run(pos, vel, L, steps, skin, reorder_interval=reorder, use_graphs=False)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+    for k in ("step", "rebuilds", "reorders", "list_entries", "max_neighbors", "max_occupancy", "ke", "pe", "virial"):
+        assert a[2][k] == b[2][k], k
+    assert np.array_equal(a[3], b[3]) and a[4] == b[4]
+    assert a[2]["rebuilds"] >= 3
+
+
+def test_run_loop_grows_its_lists_and_reports_errors():
+    pos, vel, L = state(3000, 0.6, 2.0, 52, jitter=0.05)
+    a = _run(pos, vel, L, [150], 0.4, nbr_capacity=12)
+    b = _run(pos, vel, L, [150], 0.4)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+    assert a[2]["nbr_capacity"] > 12 and a[2]["step"] == b[2]["step"] == 150
+    # two atoms thrown at each other until the force leaves its range
+    s = md.Simulation(L, 3000, RC, 0.4, DT)
+    v2 = vel.copy()
+    v2[:] *= 120.0
+    s.set_state(pos, v2)
+    with pytest.raises(md.MDError) as e:
+        s.step(200)
+    assert e.value.code == md.MD_EUNSTABLE
+    # the handle starts again from a sound state
+    s.set_state(pos, vel)
+    s.step(150)
+    p, v = s.get_state()
+    s.close()
+    assert np.array_equal(p, b[0]) and np.array_equal(v, b[1])
