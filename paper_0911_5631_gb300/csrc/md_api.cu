@@ -316,6 +316,7 @@ struct Sim : SimBase {
     int step_kernel_eager(int mode, bool final_node, cudaEvent_t after_step = nullptr) {
         cudaGraphConditionalHandle none = 0;
         int has = 0;
+        if (prm.cell_list_only) MD_CUDA(launch(cells_fn(final_node), cells_grid(), kBlock, a));
         MD_CUDA(launch(step_fn(final_node), step_grid(final_node), step_block(final_node), a, mode, none, has));
         if (after_step) {
             MD_CUDA(cudaEventRecord(after_step, stream));
@@ -324,6 +325,9 @@ struct Sim : SimBase {
         if (kStepTailNode) MD_CUDA(launch(tail_fn(final_node), 1, 32, a, mode, none, has));
         return MD_OK;
     }
+    // the cell-list-only variant's force kernel, run before its step kernel
+    void* cells_fn(bool final_node) const { return final_node ? kt.cell_forces_final : kt.cell_forces; }
+    unsigned cells_grid() const { return (unsigned)((a.n * kCellLanes + kBlock - 1) / kBlock); }
     void* tail_fn(bool final_node) const { return final_node ? kt.step_tail_final : kt.step_tail; }
 
     // ---- graphs ----------------------------------------------------------
@@ -354,22 +358,25 @@ struct Sim : SimBase {
         return cudaGraphAddNode(out, g, dep, nullptr, dep ? 1 : 0, &np);
     }
 
-    int build_body(cudaGraph_t body) {
-        int g = 0;
-        cudaGraphNode_t prev = nullptr, cur = nullptr;
-        auto chain = [&](cudaError_t e) -> cudaError_t {
-            prev = cur;
+    // Adds the rebuild branch to graph g, its first kernel after *prev (null:
+    // none); *prev becomes the last.  guard: as in rebuild_eager.
+    int add_rebuild(cudaGraph_t g, cudaGraphNode_t* prev, int guard) {
+        cudaGraphNode_t cur = nullptr;
+        bool first = *prev == nullptr;
+        auto add = [&](void* f, unsigned grid, unsigned block) -> cudaError_t {
+            cudaError_t e = add_kernel(g, first ? nullptr : prev, &cur, f, grid, block, a, guard);
+            first = false;
+            *prev = cur;
             return e;
         };
-        MD_CUDA(chain(add_kernel(body, nullptr, &cur, kt.bin, grid_atoms(), kBlock, a, g)));
-        MD_CUDA(chain(add_kernel(body, &prev, &cur, kt.scan_apply, (unsigned)a.ntiles, kBlock, a, g)));
-        MD_CUDA(chain(add_kernel(body, &prev, &cur, kt.scatter, grid_scatter(), kBlock, a, g)));
-        MD_CUDA(chain(add_kernel(body, &prev, &cur, kt.cellsort, grid_cells(), kBlock, a, g)));
-        MD_CUDA(chain(add_kernel(body, &prev, &cur, kt.gather, grid_atoms(), kBlock, a, g)));
-        MD_CUDA(chain(add_kernel(body, &prev, &cur, kt.commit, grid_atoms(), kBlock, a, g)));
-        if (!prm.cell_list_only)
-            MD_CUDA(chain(add_kernel(body, &prev, &cur, build_fn(), grid_build(), block_build(), a, g)));
-        MD_CUDA(chain(add_kernel(body, &prev, &cur, kt.rebuild_done, 1, 32, a, g)));
+        MD_CUDA(add(kt.bin, grid_atoms(), kBlock));
+        MD_CUDA(add(kt.scan_apply, (unsigned)a.ntiles, kBlock));
+        MD_CUDA(add(kt.scatter, grid_scatter(), kBlock));
+        MD_CUDA(add(kt.cellsort, grid_cells(), kBlock));
+        MD_CUDA(add(kt.gather, grid_atoms(), kBlock));
+        MD_CUDA(add(kt.commit, grid_atoms(), kBlock));
+        if (!prm.cell_list_only) MD_CUDA(add(build_fn(), grid_build(), block_build()));
+        MD_CUDA(add(kt.rebuild_done, 1, 32));
         return MD_OK;
     }
 
@@ -383,15 +390,22 @@ struct Sim : SimBase {
     // rebuild is due waits for the next conditional node.
     int build_chunk(Chunk& c, int K, bool final_node) {
         MD_CUDA(cudaGraphCreate(&c.g, 0));
-        const int m = (prm.cell_list_only || a.n > kRebuildEveryMaxAtoms) ? 1 : kRebuildEvery;
-        std::vector<cudaGraphConditionalHandle> h((K + m - 1) / m);
+        const int m = a.n > kRebuildEveryMaxAtoms ? 1 : kRebuildEvery;
+        std::vector<cudaGraphConditionalHandle> h(prm.cell_list_only ? 0 : (K + m - 1) / m);
         for (auto& hh : h) MD_CUDA(cudaGraphConditionalHandleCreate(&hh, c.g, 0, 0));
         cudaGraphNode_t prev = nullptr, node = nullptr;
-        MD_CUDA(add_kernel(c.g, nullptr, &node, kt.cond, 1, 32, a, h[0]));
-        prev = node;
+        if (!prm.cell_list_only) {
+            MD_CUDA(add_kernel(c.g, nullptr, &node, kt.cond, 1, 32, a, h[0]));
+            prev = node;
+        }
         int mode = kModeAuto;
         for (int s = 0; s < K; s++) {
-            if (s % m == 0) {
+            if (prm.cell_list_only) {
+                int r = add_rebuild(c.g, &prev, 1);
+                if (r) return r;
+                MD_CUDA(add_kernel(c.g, &prev, &node, cells_fn(final_node), cells_grid(), kBlock, a));
+                prev = node;
+            } else if (s % m == 0) {
                 NodeParams buf;
                 cudaGraphNodeParams& cp = buf.get();
                 cp.type = cudaGraphNodeTypeConditional;
@@ -400,11 +414,12 @@ struct Sim : SimBase {
                 cp.conditional.size = 1;
                 cudaGraphNode_t ifn = nullptr;
                 MD_CUDA(cudaGraphAddNode(&ifn, c.g, &prev, nullptr, 1, &cp));
-                int r = build_body(cp.conditional.phGraph_out[0]);
+                cudaGraphNode_t none = nullptr;
+                int r = add_rebuild(cp.conditional.phGraph_out[0], &none, 0);
                 if (r) return r;
                 prev = ifn;
             }
-            const int has = (s + 1 < K && (s + 1) % m == 0) ? 1 : 0;
+            const int has = (!prm.cell_list_only && s + 1 < K && (s + 1) % m == 0) ? 1 : 0;
             cudaGraphConditionalHandle nxt = has ? h[(s + 1) / m] : 0;
             MD_CUDA(add_kernel(c.g, &prev, &node, step_fn(final_node), step_grid(final_node), step_block(final_node),
                                a, mode, nxt, has));
@@ -431,7 +446,7 @@ struct Sim : SimBase {
         for (int64_t b = 0; b < count; b++) {
             MD_CUDA(cudaGraphLaunch(c.e, stream));
             graph_launches++;
-            launches += 1 + K * (kStepTailNode ? 2 : 1);
+            launches += (prm.cell_list_only ? K : 1) + K * (kStepTailNode ? 2 : 1);
         }
         return MD_OK;
     }

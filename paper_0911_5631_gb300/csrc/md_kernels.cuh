@@ -779,48 +779,145 @@ __device__ __forceinline__ void forces_mixed(const Args<Mixed>& a, int cnt, cons
     }
 }
 
-// Forces on atom i straight from the 27 cells around its cell (cell-list
-// only variant).  Candidates come from the cell-ordered copy; their pair
-// coordinates are read from the current buffer (FP64 form) or the copy
-// itself (mixed form, where the two hold the same numbers).
+// Forces straight from the 27 cells around each atom's cell (cell-list-only
+// variant), kCellLanes lanes per atom; the atoms are taken in cell order.
+// They go to fx, fy, fz, and with kEnergy the atom's halves of U and W to
+// s_ox and s_oy (scratch of the reorder, free by then); k_step integrates.
+//
+// What bounds it for small systems is one thread's chain of dependent loads
+// and, in the FP64 form, the FP64 pipe, so the lanes deal out the 27 cells,
+// and the FP64 form tests candidates in FP32 on the cell-ordered copy (the
+// bound rn2_hi is above r_c^2 by far more than that copy's rounding), queues
+// the survivors and evaluates them one per lane, as md_forces_noalloc does.
+// A thread per atom in the step kernel took 112 us for 2048 atoms.
+//
+// Mixed form: the copy holds the pair coordinates themselves and the lanes'
+// integer sums add up to the same bits in any split.
 template <class P, bool kEnergy>
-__device__ __forceinline__ void forces_from_cells(const Args<P>& a, int i, typename P::real qx,
-                                                  typename P::real qy, typename P::real qz,
-                                                  const typename P::pos4* __restrict__ pc,
-                                                  typename AccOf<P>::type& acc) {
+__global__ void __launch_bounds__(kBlock) k_cell_forces(Args<P> a) {
     using real = typename P::real;
+    using Acc = typename AccOf<P>::type;
+    constexpr unsigned kFull = 0xffffffffu;
+    constexpr int kQueue = 16;   // survivors an atom queues (FP64 form)
+    constexpr int kCells = (27 + kCellLanes - 1) / kCellLanes;  // cells of a lane
+    constexpr int kFirst = 2;    // candidates of a cell loaded ahead (a cell holds about one)
+    static_assert(kCellLanes == 8, "the queue's bookkeeping");
+    __shared__ int s_queue[P::kFp64 ? kBlock / kCellLanes * kQueue : 1];
+    const int lane = threadIdx.x & 31, sub = lane % kCellLanes, shift = lane - sub;
+    const unsigned below = (1u << sub) - 1u;
+    const int64_t s = gtid() / kCellLanes;
+    const bool in = s < a.n;
+    const float4 ci = a.cand[in ? s : 0];
+    const int i = __float_as_int(ci.w);
     int cx, cy, cz;
     unpack_cell(a.cell[i], cx, cy, cz);
-    real wx, wy, wz;
-    if constexpr (P::kFp64) { wx = a.w[0]; wy = a.w[1]; wz = a.w[2]; }
-    else { wx = a.wf[0]; wy = a.wf[1]; wz = a.wf[2]; }
-    for (int dz = -1; dz <= 1; dz++) {
-        int z = wrap_add(cz, dz, a.G[2]);
-        real sz = -(real)dz * wz;
-        for (int dy = -1; dy <= 1; dy++) {
-            int y = wrap_add(cy, dy, a.G[1]);
-            real sy = -(real)dy * wy;
-            for (int dx = -1; dx <= 1; dx++) {
-                int x = wrap_add(cx, dx, a.G[0]);
-                real sx = -(real)dx * wx;
-                int c2 = cell_index(x, y, z, a.G);
-                int beg = a.cell_start[c2], end = min(a.cell_start[c2 + 1], (int)a.n);
-                for (int t = beg; t < end; t++) {
-                    float4 cj = __ldg(a.cand + t);
-                    int j = __float_as_int(cj.w);
-                    if (j == i) continue;
-                    real px, py, pz;
-                    if constexpr (P::kFp64) {
-                        auto pj = ld_pos4(pc + min((unsigned)j, (unsigned)(a.n - 1)));
-                        px = pj.x; py = pj.y; pz = pj.z;
-                    } else {
-                        px = cj.x; py = cj.y; pz = cj.z;
-                    }
-                    acc.template pair<kEnergy>(a, (qx - px) + sx, (qy - py) + sy, (qz - pz) + sz);
-                }
-            }
+    const typename P::pos4* pc = a.ctr->parity ? a.pB : a.pA;
+    const typename P::pos4 qi = ld_pos4(pc + i);
+    int* queue = s_queue + (P::kFp64 ? (int)(threadIdx.x / kCellLanes) * kQueue : 0);
+    Acc acc;
+    int nq = 0;
+
+    auto evaluate = [&]() {  // (FP64 form) the queued pairs, one a lane
+        __syncwarp();
+        for (int p = sub; __any_sync(kFull, p < nq); p += kCellLanes) {
+            if (p >= nq) continue;
+            const unsigned e = (unsigned)queue[p];
+            const auto pj = ld_pos4(pc + (e & a.jmask));
+            const unsigned c = e >> kCodeShift;
+            const real dx = (qi.x - pj.x) + (real)(1 - (int)(c & 3u)) * (real)a.w[0];
+            const real dy = (qi.y - pj.y) + (real)(1 - (int)((c >> 2) & 3u)) * (real)a.w[1];
+            const real dz = (qi.z - pj.z) + (real)(1 - (int)(c >> 4)) * (real)a.w[2];
+            const real r2 = acc.r2(dx, dy, dz);
+            if (acc.inside(a, r2)) acc.template force<kEnergy>(a, dx, dy, dz, r2);
+        }
+        __syncwarp();
+        nq = 0;
+    };
+    // one candidate of stencil cell d (lanes without one: have = false)
+    auto test = [&](const float4& cj, bool have, int d) {
+        const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
+        const int j = __float_as_int(cj.w);
+        const float ex = (ci.x - cj.x) + -(float)dx * a.wf[0];
+        const float ey = (ci.y - cj.y) + -(float)dy * a.wf[1];
+        const float ez = (ci.z - cj.z) + -(float)dz * a.wf[2];
+        if constexpr (P::kFp64) {
+            const bool keep = have && j != i && fmaf(ex, ex, fmaf(ey, ey, ez * ez)) < a.rn2_hi;
+            const unsigned m = (__ballot_sync(kFull, keep) >> shift) & ((1u << kCellLanes) - 1u);
+            if (keep) queue[nq + __popc(m & below)] = j | (((dx + 1) | ((dy + 1) << 2) | ((dz + 1) << 4)) << kCodeShift);
+            nq += __popc(m);
+            if (__any_sync(kFull, nq > kQueue - kCellLanes)) evaluate();
+        } else {
+            if (have && j != i) acc.template pair<kEnergy>(a, ex, ey, ez);
+        }
+    };
+
+    int lo[kCells], hi[kCells];
+#pragma unroll
+    for (int q = 0; q < kCells; q++) {
+        const int d = sub + kCellLanes * q;
+        lo[q] = hi[q] = 0;
+        if (d < 27 && in) {
+            const int c = cell_index(wrap_add(cx, d % 3 - 1, a.G[0]), wrap_add(cy, (d / 3) % 3 - 1, a.G[1]),
+                                     wrap_add(cz, d / 9 - 1, a.G[2]), a.G);
+            lo[q] = a.cell_start[c];
+            hi[q] = min(a.cell_start[c + 1], (int)a.n);
         }
     }
+    float4 first[kCells][kFirst];
+#pragma unroll
+    for (int q = 0; q < kCells; q++)
+#pragma unroll
+        for (int u = 0; u < kFirst; u++)
+            first[q][u] = lo[q] + u < hi[q] ? __ldg(a.cand + lo[q] + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < kCells; q++) {
+        const int d = sub + kCellLanes * q;
+#pragma unroll
+        for (int u = 0; u < kFirst; u++) test(first[q][u], lo[q] + u < hi[q], d);
+        for (int t = lo[q] + kFirst; __any_sync(kFull, t < hi[q]); t++)
+            test(t < hi[q] ? __ldg(a.cand + t) : make_float4(0.f, 0.f, 0.f, 0.f), t < hi[q], d);
+    }
+    if constexpr (P::kFp64) evaluate();
+
+    // the sums over the atom's lanes
+    if constexpr (P::kFp64) {
+#pragma unroll
+        for (int w = 1; w < kCellLanes; w <<= 1) {
+            acc.fx += __shfl_xor_sync(kFull, acc.fx, w);
+            acc.fy += __shfl_xor_sync(kFull, acc.fy, w);
+            acc.fz += __shfl_xor_sync(kFull, acc.fz, w);
+            if constexpr (kEnergy) {
+                acc.u += __shfl_xor_sync(kFull, acc.u, w);
+                acc.w += __shfl_xor_sync(kFull, acc.w, w);
+            }
+        }
+    } else {
+        auto total = [&](Fix& f) {
+#pragma unroll
+            for (int w = 1; w < kCellLanes; w <<= 1) {
+                f.a += __shfl_xor_sync(kFull, f.a, w);
+                f.b += __shfl_xor_sync(kFull, f.b, w);
+                f.c += __shfl_xor_sync(kFull, f.c, w);
+            }
+        };
+        total(acc.fxy.x);
+        total(acc.fxy.y);
+        total(acc.fz);
+        if constexpr (kEnergy) {
+            total(acc.u);
+            total(acc.w);
+        }
+    }
+    if (in && sub == 0) {
+        a.fx[i] = acc.force_x();
+        a.fy[i] = acc.force_y();
+        a.fz[i] = acc.force_z();
+        if constexpr (kEnergy) {
+            a.s_ox[i] = 0.5 * acc.energy();
+            a.s_oy[i] = 0.5 * acc.virial();
+        }
+    }
+    if (__any_sync(kFull, in && acc.close) && lane == 0) atomicOr(&a.ctr->close_flag, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -1870,26 +1967,33 @@ __device__ __forceinline__ void step_atom(const Args<P>& a, int64_t i, bool in, 
     constexpr bool kTogether = P::kFp64 && !kCells;
     if (!active || !(in || kTogether)) return;
     {
-        const pos4 qi = ld_pos4(pc + (in ? i : 0));
-        const real qx = qi.x, qy = qi.y, qz = qi.z;
         typename AccOf<P>::type acc;
         if constexpr (kTogether) {
-            forces_fp64<kFinal, f64_results(kFinal)>(a, in ? cnt : 0, col, rows, staged, qx, qy, qz,
+            const pos4 qi = ld_pos4(pc + (in ? i : 0));
+            forces_fp64<kFinal, f64_results(kFinal)>(a, in ? cnt : 0, col, rows, staged, qi.x, qi.y, qi.z,
                                                      (unsigned long long)__double_as_longlong(qi.w), pc, f64_tab,
                                                      f64_res, acc);
             if (!in) {
                 close = acc.close != 0;
                 return;
             }
-        } else if (kFinal && energy) {
-            if constexpr (kCells) forces_from_cells<P, kFinal>(a, (int)i, qx, qy, qz, pc, acc);
-            else forces_mixed<kFinal, kLdg, kRows>(a, cnt, col, rows, staged, qx, qy, qz, pc, acc);
-        } else {
-            if constexpr (kCells) forces_from_cells<P, false>(a, (int)i, qx, qy, qz, pc, acc);
+        } else if constexpr (!kCells) {
+            const pos4 qi = ld_pos4(pc + i);
+            const real qx = qi.x, qy = qi.y, qz = qi.z;
+            if (kFinal && energy) forces_mixed<kFinal, kLdg, kRows>(a, cnt, col, rows, staged, qx, qy, qz, pc, acc);
             else forces_mixed<false, kLdg, kRows>(a, cnt, col, rows, staged, qx, qy, qz, pc, acc);
         }
         close = acc.close != 0;
-        real fx = acc.force_x(), fy = acc.force_y(), fz = acc.force_z();
+        real fx, fy, fz;
+        if constexpr (kCells) {  // k_cell_forces
+            fx = a.fx[i];
+            fy = a.fy[i];
+            fz = a.fz[i];
+        } else {
+            fx = acc.force_x();
+            fy = acc.force_y();
+            fz = acc.force_z();
+        }
         vel vx = a.vx[i], vy = a.vy[i], vz = a.vz[i];
         const real pbx = a.pbx[i], pby = a.pby[i], pbz = a.pbz[i];
         double ox = a.ox[i], oy = a.oy[i], oz = a.oz[i];
@@ -1899,13 +2003,13 @@ __device__ __forceinline__ void step_atom(const Args<P>& a, int64_t i, bool in, 
             vz = kick(a, vz, fz);
         }
         if (energy) {
-            a.fx[i] = fx; a.fy[i] = fy; a.fz[i] = fz;
+            if constexpr (!kCells) { a.fx[i] = fx; a.fy[i] = fy; a.fz[i] = fz; }
             double dvx, dvy, dvz;
             if constexpr (P::kFp64) { dvx = vx; dvy = vy; dvz = vz; }
             else { dvx = cvt::f64(vx); dvy = cvt::f64(vy); dvz = cvt::f64(vz); }
             ke = 0.5 * (dvx * dvx + dvy * dvy + dvz * dvz);
-            pe = 0.5 * acc.energy();
-            vir = 0.5 * acc.virial();
+            pe = kCells ? a.s_ox[i] : 0.5 * acc.energy();
+            vir = kCells ? a.s_oy[i] : 0.5 * acc.virial();
             if (!init) { a.vx[i] = vx; a.vy[i] = vy; a.vz[i] = vz; }
         } else {
             vx = kick(a, vx, fx);
@@ -2664,6 +2768,8 @@ KernelTable<P> make_kernel_table() {
     if constexpr (P::kFp64) t.step_list = (void*)k_step<P, false, false, kStepBlockF64>;
     else t.step_list = (void*)k_step<P, false, false, kStepBlockMixed>;
     t.step_list_final = (void*)k_step<P, false, true>;
+    t.cell_forces = (void*)k_cell_forces<P, false>;
+    t.cell_forces_final = (void*)k_cell_forces<P, true>;
     t.step_cells = (void*)k_step<P, true, false>;
     t.step_cells_final = (void*)k_step<P, true, true>;
     t.finalize = (void*)k_finalize<P>;

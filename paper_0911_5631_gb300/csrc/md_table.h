@@ -25,6 +25,8 @@ struct KernelTable {
     void* step_tail_final;
     void* step_list;
     void* step_list_final;
+    void* cell_forces;        // cell-list-only forces, before step_cells
+    void* cell_forces_final;  // the same with energies
     void* step_cells;
     void* step_cells_final;
     void* finalize;
