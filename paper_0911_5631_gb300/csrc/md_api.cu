@@ -245,6 +245,7 @@ struct Sim : SimBase {
     }
 
     unsigned grid_atoms() const { return (unsigned)a.nblocks; }
+    static unsigned few(unsigned blocks) { return std::min(blocks, 8u * 152u); }  // eight blocks on an SM
     unsigned grid_cells() const { return (unsigned)((a.ncells + kBlock - 1) / kBlock); }
     unsigned grid_scatter() const {
         int64_t m = a.n > a.ncells ? a.n : a.ncells;
@@ -299,9 +300,8 @@ struct Sim : SimBase {
         MD_CUDA(launch(kt.bin, grid_atoms(), kBlock, a, g));
         MD_CUDA(launch(kt.scan_apply, (unsigned)a.ntiles, kBlock, a, g));
         MD_CUDA(launch(kt.scatter, grid_scatter(), kBlock, a, g));
-        MD_CUDA(launch(kt.cellsort, grid_cells(), kBlock, a, g));
-        MD_CUDA(launch(kt.gather, grid_atoms(), kBlock, a, g));
-        MD_CUDA(launch(kt.commit, grid_atoms(), kBlock, a, g));
+        MD_CUDA(launch(kt.sort_gather, few(grid_cells()), kBlock, a, g));
+        MD_CUDA(launch(kt.commit, few(grid_atoms()), kBlock, a, g));
         if (!prm.cell_list_only) MD_CUDA(launch(build_fn(), grid_build(), block_build(), a, g));
         MD_CUDA(launch(kt.rebuild_done, 1, 32, a, g));
         return MD_OK;
@@ -372,9 +372,8 @@ struct Sim : SimBase {
         MD_CUDA(add(kt.bin, grid_atoms(), kBlock));
         MD_CUDA(add(kt.scan_apply, (unsigned)a.ntiles, kBlock));
         MD_CUDA(add(kt.scatter, grid_scatter(), kBlock));
-        MD_CUDA(add(kt.cellsort, grid_cells(), kBlock));
-        MD_CUDA(add(kt.gather, grid_atoms(), kBlock));
-        MD_CUDA(add(kt.commit, grid_atoms(), kBlock));
+        MD_CUDA(add(kt.sort_gather, few(grid_cells()), kBlock));
+        MD_CUDA(add(kt.commit, few(grid_atoms()), kBlock));
         if (!prm.cell_list_only) MD_CUDA(add(build_fn(), grid_build(), block_build()));
         MD_CUDA(add(kt.rebuild_done, 1, 32));
         return MD_OK;
@@ -889,7 +888,7 @@ struct Sim : SimBase {
         if (r) return r;
         std::memset(out, 0, sizeof(*out));
         // every rebuild branch that ran launched its kernels
-        int per_rebuild = prm.cell_list_only ? 7 : 8;
+        const int per_rebuild = prm.cell_list_only ? 6 : 7;
         int64_t body = prm.use_graphs && !profiling ? (int64_t)(c.rebuilds - c.run_rebuilds) * per_rebuild : 0;
         out->launches = launches + body;
         out->step_kernel_launches = step_launches;

@@ -191,6 +191,7 @@ struct alignas(16) Args {
     double w[3];        // cell widths
     double hw[3];       // half cell widths
     float hwf_in[3];    // FP32 bound below which an offset is surely inside its cell
+    float hwf_out[3];   // FP32 bound above which it is surely outside
     unsigned jmask;     // pair_slots(n) - 1: masks a list entry to its index (below n for every
                         // entry a build writes) and keeps any masked index inside pA / pB
     double hw_in[3];    // FP64 bound below which the whole-cell moves of a re-binning are exact

@@ -139,6 +139,7 @@ void fill_args_scalars(Args<P>& a, const md_plan_t& plan, const double box[3], i
         a.w[k] = plan.w[k];
         a.hw[k] = 0.5 * plan.w[k];
         a.hwf_in[k] = (float)(0.5 * plan.w[k] * (1.0 - 1e-6));
+        a.hwf_out[k] = (float)(0.5 * plan.w[k] * (1.0 + 1e-6));
         a.hw_in[k] = 0.5 * plan.w[k] * (1.0 - 1e-9);
         a.wf[k] = (float)plan.w[k];
         const double periods = std::fmax(1.0, std::floor(box[k] / (3.0 * (rc + skin))));

@@ -1026,15 +1026,30 @@ __device__ __forceinline__ int bin_item(const Args<P>& a, int64_t i, int parity)
         // offset closer to a face, or an atom more than two cells away, is
         // binned by the rule itself from the reported position.
         if (!(fabsf(to_f32(pb[d])) < a.hwf_in[d])) {
-            double tn = t;
-            int c = cc[d];
-            for (int it = 0; it < 2; it++) {
-                if (tn >= a.hw[d]) { tn = __dsub_rn(tn, a.w[d]); c = wrap_add(c, 1, a.G[d]); }
-                else if (tn < -a.hw[d]) { tn = __dadd_rn(tn, a.w[d]); c = wrap_add(c, -1, a.G[d]); }
+            // An offset clearly outside that lies clearly inside the next
+            // cell needs one FP64 operation for the move (the comparisons
+            // above would run on the FP64 pipe, which bounds the binning, and
+            // nearly every warp has such an atom).
+            const float f = to_f32(pb[d]);
+            const bool out = fabsf(f) > a.hwf_out[d];
+            double tn = out ? __dadd_rn(t, f > 0.0f ? -a.w[d] : a.w[d]) : t;
+            int c = out ? wrap_add(cc[d], f > 0.0f ? 1 : -1, a.G[d]) : cc[d];
+            real pn;
+            double on;
+            split_offset(tn, pn, on);
+            if (!(out && fabsf(to_f32(pn)) < a.hwf_in[d])) {
+                tn = t;
+                c = cc[d];
+                for (int it = 0; it < 2; it++) {
+                    if (tn >= a.hw[d]) { tn = __dsub_rn(tn, a.w[d]); c = wrap_add(c, 1, a.G[d]); }
+                    else if (tn < -a.hw[d]) { tn = __dadd_rn(tn, a.w[d]); c = wrap_add(c, -1, a.G[d]); }
+                }
+                if (!(fabs(tn) < a.hw_in[d])) bad |= !bin_coord(a, d, abs_coord(a, d, cc[d], t), c, tn);
+                split_offset(tn, pn, on);
             }
-            if (!(fabs(tn) < a.hw_in[d])) bad |= !bin_coord(a, d, abs_coord(a, d, cc[d], t), c, tn);
             cc[d] = c;
-            split_offset(tn, pb[d], o[d]);
+            pb[d] = pn;
+            o[d] = on;
         }
         pbp[d][i] = pb[d];
         op[d][i] = o[d];
@@ -1116,23 +1131,39 @@ __global__ void __launch_bounds__(kBlock) k_scan_apply(Args<P> a, int guard) {
     if (threadIdx.x == 0) atomicMax(&C->max_occ, bm);
 }
 
-// Places each atom at cell_start[cell] + rank (the cell's arrival order)
-// and clears the counts for the next binning.
+// Whether a rebuild sorts each cell's atoms.  The FP64 form always does: its
+// force sums depend on the order of the lists.  Nothing in the mixed form
+// depends on the order inside a cell but the storage order that a reorder
+// gives the atoms, so between reorders a cell's atoms keep their order of
+// arrival, and the scatter writes the candidates itself.
 template <class P>
-__device__ __forceinline__ int scatter_item(const Args<P>& a, int64_t t) {
-    const int slot = a.cell_start[cell_index_of_packed(a.cell[t], a.G)] + a.rank[t];
-    if (slot >= 0 && slot < a.n) {
-        a.order[slot] = (int)t;
-        return slot;
-    }
-    atomicOr(&a.ctr->error, kErrUnstable);
-    return -1;
+__device__ __forceinline__ bool sorts_cells(int reorder) {
+    return P::kFp64 || reorder;
 }
 
+// The candidate that an atom is to the neighbour search: its FP32 coordinates
+// in its cell and its storage index.  Right after a binning the displacement
+// is what FP32 left of the offset (or 0), so pb is the coordinate.
+template <class P>
+__device__ __forceinline__ float4 candidate(const Args<P>& a, int64_t i, int index) {
+    return make_float4(to_f32(a.pbx[i]), to_f32(a.pby[i]), to_f32(a.pbz[i]), __int_as_float(index));
+}
+
+// Places each atom at cell_start[cell] + rank (the cell's arrival order).
+template <class P>
+__device__ __forceinline__ void scatter_item(const Args<P>& a, int64_t t, int reorder) {
+    const int slot = a.cell_start[cell_index_of_packed(a.cell[t], a.G)] + a.rank[t];
+    if (slot < 0 || slot >= a.n) atomicOr(&a.ctr->error, kErrUnstable);
+    else if (sorts_cells<P>(reorder)) a.order[slot] = (int)t;
+    else a.cand[slot] = candidate(a, t, (int)t);
+}
+
+// ... and clears the counts for the next binning.
 template <class P>
 __global__ void __launch_bounds__(kBlock) k_scatter(Args<P> a, int guard) {
     if (guard && !a.ctr->rebuild_flag) return;
-    for (int64_t t = gtid(); t < a.n; t += (int64_t)gridDim.x * blockDim.x) scatter_item<P>(a, t);
+    const int reorder = a.ctr->reorder_now;
+    for (int64_t t = gtid(); t < a.n; t += (int64_t)gridDim.x * blockDim.x) scatter_item<P>(a, t, reorder);
     // counts and tile totals are no longer needed once cell_start is known
     for (int64_t t = gtid(); t < a.ncells; t += (int64_t)gridDim.x * blockDim.x) a.count[t] = 0;
     for (int64_t t = gtid(); t < a.ntiles; t += (int64_t)gridDim.x * blockDim.x) a.tile_sum[t] = 0;
@@ -1176,41 +1207,35 @@ __device__ __forceinline__ void cellsort_item(const Args<P>& a, int64_t c) {
     }
 }
 
-template <class P>
-__global__ void __launch_bounds__(kBlock) k_cellsort(Args<P> a, int guard) {
-    if (guard && !a.ctr->rebuild_flag) return;
-    int64_t c = gtid();
-    if (c >= a.ncells) return;
-    cellsort_item<P>(a, c);
-}
-
 // Writes the cell-ordered FP32 coordinate copy used by the neighbour search
 // and, when a reorder is due, the state permuted into cell order (Sec. 3.5).
 template <class P>
 __device__ __forceinline__ void gather_item(const Args<P>& a, int64_t s, int reorder) {
-    using real = typename P::real;
-    int i = a.order[s];
-    real pbx = a.pbx[i], pby = a.pby[i], pbz = a.pbz[i];
-    double ox = a.ox[i], oy = a.oy[i], oz = a.oz[i];
-    real px = pair_coord(pbx, ox), py = pair_coord(pby, oy), pz = pair_coord(pbz, oz);
-    a.cand[s] = make_float4(to_f32(px), to_f32(py), to_f32(pz), __int_as_float(reorder ? (int)s : i));
+    const int i = a.order[s];
+    a.cand[s] = candidate(a, i, reorder ? (int)s : i);
     if (reorder) {
         a.s_cell[s] = a.cell[i];
         a.s_perm[s] = a.perm[i];
-        a.s_pbx[s] = pbx; a.s_pby[s] = pby; a.s_pbz[s] = pbz;
-        a.s_ox[s] = ox; a.s_oy[s] = oy; a.s_oz[s] = oz;
+        a.s_pbx[s] = a.pbx[i]; a.s_pby[s] = a.pby[i]; a.s_pbz[s] = a.pbz[i];
+        a.s_ox[s] = a.ox[i]; a.s_oy[s] = a.oy[i]; a.s_oz[s] = a.oz[i];
         a.s_vx[s] = a.vx[i]; a.s_vy[s] = a.vy[i]; a.s_vz[s] = a.vz[i];
     }
 }
 
+// Sorts and gathers each cell, a thread per cell.  Most rebuilds of the mixed
+// form have neither to do, and 4096 blocks that return at once take 5 us, so
+// this kernel and k_commit run few blocks that stride.
 template <class P>
-__global__ void __launch_bounds__(kBlock) k_gather(Args<P> a, int guard) {
-    using real = typename P::real;
-    Counters* C = a.ctr;
+__global__ void __launch_bounds__(kBlock) k_sort_gather(Args<P> a, int guard) {
+    const Counters* C = a.ctr;
     if (guard && !C->rebuild_flag) return;
-    int64_t s = gtid();
-    if (s >= a.n) return;
-    gather_item<P>(a, s, C->reorder_now);
+    const int reorder = C->reorder_now;
+    if (!sorts_cells<P>(reorder)) return;
+    for (int64_t c = gtid(); c < a.ncells; c += (int64_t)gridDim.x * blockDim.x) {
+        cellsort_item<P>(a, c);
+        const int end = min(a.cell_start[c + 1], (int)a.n);
+        for (int s = a.cell_start[c]; s < end; s++) gather_item<P>(a, s, reorder);
+    }
 }
 
 // Copies the permuted state back and rewrites the current pair buffer in
@@ -1234,9 +1259,8 @@ __global__ void __launch_bounds__(kBlock) k_commit(Args<P> a, int guard) {
     Counters* C = a.ctr;
     if (guard && !C->rebuild_flag) return;
     if (!C->reorder_now) return;
-    int64_t s = gtid();
-    if (s >= a.n) return;
-    commit_item<P>(a, s, C->parity);
+    const int parity = C->parity;
+    for (int64_t s = gtid(); s < a.n; s += (int64_t)gridDim.x * blockDim.x) commit_item<P>(a, s, parity);
 }
 
 // Exact FP64 neighbour criterion r^2 < r_n^2 for atom i and atom j, whose
@@ -1292,6 +1316,35 @@ __device__ __forceinline__ int shell_reach(const Args<P>& a, unsigned d2bits) {
     if (!a.shell_bins) return kShellBins;
     const float t = fmaf(2.0f, sqrtf(__uint_as_float(d2bits)), a.shell_eps) * a.shell_inv;
     return t < (float)(kShellBins - 1) ? max((int)ceilf(t), 1) : kShellBins;
+}
+
+// Closes a rebuild: counters, reorder bookkeeping, flag cleared, and the
+// running maximum of the displacement restarted.  One warp.
+template <class P>
+__device__ __forceinline__ void rebuild_done(const Args<P>& a) {
+    Counters* C = a.ctr;
+    if (a.d2b)
+        for (int b = threadIdx.x & 31; b < kD2Buckets; b += 32) a.d2b[b * 32] = 0u;
+    if ((threadIdx.x & 31) != 0) return;
+    C->rebuilds += 1;
+    if (C->reorder_now) {
+        C->reorders += 1;
+        C->since_reorder = 0;
+        C->reorder_now = 0;
+    }
+    C->rebuild_flag = 0;
+    C->d2max = 0u;  // displacements now count from the new build
+    C->reach = shell_reach(a, 0u);
+}
+
+// (A node of its own: the last block of the build doing it by an atomic
+// ticket made the build 6 us longer at 1M atoms.)
+template <class P>
+__global__ void k_rebuild_done(Args<P> a, int guard) {
+    if (blockIdx.x != 0 || threadIdx.x >= 32) return;
+    const bool run = !guard || a.ctr->rebuild_flag;
+    __syncwarp();  // every lane has read the flag before lane 0 clears it
+    if (run) rebuild_done(a);
 }
 
 // Neighbour-list build (Sec. 3.4): for the atom in cell-ordered slot s, scan
@@ -1764,29 +1817,6 @@ __global__ void __launch_bounds__(kWcThreads, 2) k_build_wc(Args<P> a, int guard
         atomicMax(&C->max_nn, bm);
         atomicAdd((unsigned long long*)&C->list_entries, (unsigned long long)bs);
     }
-}
-
-// Closes a rebuild: counters, reorder bookkeeping, flag cleared, and the
-// running maximum of the displacement restarted.  One warp.
-template <class P>
-__global__ void k_rebuild_done(Args<P> a, int guard) {
-    Counters* C = a.ctr;
-    if (blockIdx.x != 0 || threadIdx.x >= 32) return;
-    const bool run = !guard || C->rebuild_flag;
-    __syncwarp();  // every lane has read the flag before lane 0 clears it
-    if (!run) return;
-    if (a.d2b)
-        for (int b = threadIdx.x; b < kD2Buckets; b += 32) a.d2b[b * 32] = 0u;
-    if (threadIdx.x != 0) return;
-    C->rebuilds += 1;
-    if (C->reorder_now) {
-        C->reorders += 1;
-        C->since_reorder = 0;
-        C->reorder_now = 0;
-    }
-    C->rebuild_flag = 0;
-    C->d2max = 0u;  // displacements now count from the new build
-    C->reach = shell_reach(a, 0u);
 }
 
 // Graph prologue: copies the device rebuild flag into the first
@@ -2479,14 +2509,15 @@ __device__ __noinline__ void ens_rebuild(const Args<P>& a, EnsShared& sh, int* s
     tm.sync();
     if (tm.lead_block()) ens_scan<P>(a, sh);
     tm.sync();
-    for (int64_t t = t0; t < n; t += dt) scatter_item<P>(a, t);
+    const int reorder = C->reorder_now;
+    for (int64_t t = t0; t < n; t += dt) scatter_item<P>(a, t, reorder);
     for (int64_t c = t0; c < a.ncells; c += dt) a.count[c] = 0;
     tm.sync();
-    for (int64_t c = t0; c < a.ncells; c += dt) cellsort_item<P>(a, c);
-    tm.sync();
-    for (int64_t s = t0; s < n; s += dt) gather_item<P>(a, s, C->reorder_now);
-    tm.sync();
-    if (C->reorder_now) {
+    if (reorder) {
+        for (int64_t c = t0; c < a.ncells; c += dt) cellsort_item<P>(a, c);
+        tm.sync();
+        for (int64_t s = t0; s < n; s += dt) gather_item<P>(a, s, reorder);
+        tm.sync();
         for (int64_t s = t0; s < n; s += dt) commit_item<P>(a, s, C->parity);
         tm.sync();
     }
@@ -2753,8 +2784,7 @@ KernelTable<P> make_kernel_table() {
     t.bin = (void*)k_bin<P>;
     t.scan_apply = (void*)k_scan_apply<P>;
     t.scatter = (void*)k_scatter<P>;
-    t.cellsort = (void*)k_cellsort<P>;
-    t.gather = (void*)k_gather<P>;
+    t.sort_gather = (void*)k_sort_gather<P>;
     t.commit = (void*)k_commit<P>;
     t.build = (void*)k_build<P>;
     t.build_rows = (void*)k_build<P, true>;

@@ -141,7 +141,9 @@ __device__ __noinline__ bool run_within_rn(const Args<P>& a, int i, int j, unsig
 // entries of all four are written out ordered by shell bin.  Returns the
 // atom's entry count in every lane.  Every lane of the warp must call it (in =
 // false: no atom).
-template <class P>
+// kRowsAhead: rows whose loads are issued together (fewer where registers are
+// short: a spilled one costs a trip to L2 after each barrier).
+template <class P, int kRowsAhead>
 __device__ __forceinline__ int run_build(const Args<P>& a, int64_t s, bool in, int2* stage, int stride) {
     constexpr unsigned kFull = 0xffffffffu;
     constexpr int kEach = 3;  // candidates of a row that a lane loads ahead: 12 per row
@@ -187,11 +189,11 @@ __device__ __forceinline__ int run_build(const Args<P>& a, int64_t s, bool in, i
     }
     const float qx0 = ci.x + a.wf[0], qx1 = ci.x, qx2 = ci.x - a.wf[0];  // x seen from cells x-1, x, x+1
 #pragma unroll
-    for (int r0 = 0; r0 < 9; r0 += 3) {
-        int m0[3], m1[3], m2[3], s0[3], s1[3], s2[3];
-        float4 pj[3][kEach];
+    for (int r0 = 0; r0 < 9; r0 += kRowsAhead) {
+        int m0[kRowsAhead], m1[kRowsAhead], m2[kRowsAhead], s0[kRowsAhead], s1[kRowsAhead], s2[kRowsAhead];
+        float4 pj[kRowsAhead][kEach];
 #pragma unroll
-        for (int w = 0; w < 3; w++) {
+        for (int w = 0; w < kRowsAhead; w++) {
             const int r = r0 + w, q = r / kRunLanes, from = lead + r % kRunLanes;
             m0[w] = __shfl_sync(kFull, n0[q], from);
             m1[w] = __shfl_sync(kFull, n1[q], from);
@@ -206,7 +208,7 @@ __device__ __forceinline__ int run_build(const Args<P>& a, int64_t s, bool in, i
             }
         }
 #pragma unroll
-        for (int w = 0; w < 3; w++) {
+        for (int w = 0; w < kRowsAhead; w++) {
             const int r = r0 + w, dy = r % 3 - 1, dz = r / 3 - 1;
             const float qz = ci.z - (float)dz * a.wf[2];
             const float qy = ci.y - (float)dy * a.wf[1];
@@ -318,12 +320,7 @@ __device__ __noinline__ int run_rebuild(const Args<P>& a, int64_t i, int par, in
     for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) run_scan_tile(a, t, s_scan);
     said |= bar.sync(0, s_sync, C);
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, dt = (int64_t)gridDim.x * blockDim.x;
-    if (in && sub == 0) {
-        const int slot = scatter_item<P>(a, i);
-        if (!reorder && slot >= 0)
-            a.cand[slot] = make_float4(pair_coord(a.pbx[i], a.ox[i]), pair_coord(a.pby[i], a.oy[i]),
-                                       pair_coord(a.pbz[i], a.oz[i]), __int_as_float((int)i));
-    }
+    if (in && sub == 0) scatter_item<P>(a, i, reorder);
     for (int64_t c = t0; c < a.ncells; c += dt) a.count[c] = 0;
     for (int64_t c = t0; c < a.ntiles; c += dt) a.tile_sum[c] = 0;
     said |= bar.sync(0, s_sync, C);
@@ -335,7 +332,7 @@ __device__ __noinline__ int run_rebuild(const Args<P>& a, int64_t i, int par, in
         if (in && sub == 0) commit_item<P>(a, i, par);
         said |= bar.sync(0, s_sync, C);
     }
-    const int m = run_build(a, i, in, stage, (int)blockDim.x);
+    const int m = run_build<P, kB == kRunMaxBlock ? 1 : 3>(a, i, in, stage, (int)blockDim.x);
     const int wmax = __reduce_max_sync(kFull, m);
     const int wsum = __reduce_add_sync(kFull, sub == 0 ? m : 0);
     if (lane == 0) {

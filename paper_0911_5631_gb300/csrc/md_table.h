@@ -11,8 +11,7 @@ struct KernelTable {
     void* bin;
     void* scan_apply;
     void* scatter;
-    void* cellsort;
-    void* gather;
+    void* sort_gather;
     void* commit;
     void* build;     // thread per atom
     void* build_rows;  // the same, lists with each atom's entries contiguous (W transposed)
