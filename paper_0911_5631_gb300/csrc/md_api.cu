@@ -589,8 +589,10 @@ struct Sim : SimBase {
             return MD_ECUDA;
         }
         if (c.error & (kErrUnstable | kErrClose)) {
-            err = (c.error & kErrClose) ? "two atoms came closer than the fixed-point force range allows"
-                                        : "non-finite coordinate or velocity";
+            // (a non-finite input is binned at its cell's centre, where it may
+            // meet another)
+            err = (c.error & kErrUnstable) ? "non-finite coordinate or velocity"
+                                           : "two atoms came closer than the fixed-point force range allows";
             return MD_EUNSTABLE;
         }
         return MD_OK;
@@ -656,6 +658,17 @@ struct Sim : SimBase {
 
     // ---- API -------------------------------------------------------------
 
+    // Whether a kernel may use the caller's array in place of a staged copy:
+    // memory of this device, aligned to its elements.
+    bool direct(const void* p) const {
+        cudaPointerAttributes at;
+        if (((uintptr_t)p & 7u) != 0 || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        return at.type == cudaMemoryTypeDevice && at.device == this->device;
+    }
+
     int set_state(const double* pos, const double* vel, bool device) override {
         DevGuard dg(this->device);
         if (!pos || !vel) {
@@ -663,32 +676,38 @@ struct Sim : SimBase {
             return MD_EINVAL;
         }
         size_t bytes = sizeof(double) * 3 * (size_t)a.n;
-        cudaMemcpyKind k = device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-        MD_CUDA(cudaMemcpyAsync(a.io_pos, pos, bytes, k, stream));
-        MD_CUDA(cudaMemcpyAsync(a.io_vel, vel, bytes, k, stream));
+        Args<P> in = a;  // reads the caller's arrays where it can
+        if (device && direct(pos) && direct(vel)) {
+            in.io_pos = const_cast<double*>(pos);
+            in.io_vel = const_cast<double*>(vel);
+        } else {
+            cudaMemcpyKind k = device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+            MD_CUDA(cudaMemcpyAsync(a.io_pos, pos, bytes, k, stream));
+            MD_CUDA(cudaMemcpyAsync(a.io_vel, vel, bytes, k, stream));
+        }
         MD_CUDA(launch(kt.reset_counters, 1, 32, a.ctr));
-        MD_CUDA(launch(kt.set_state, grid_atoms(), kBlock, a));
+        MD_CUDA(launch(kt.set_state, grid_atoms(), kBlock, in));
         int r = rebuild_eager();
         if (r) return r;
+        // the forces follow at once; a list that turns out to have overflowed
+        // is grown and they are computed again
         for (int attempt = 0; attempt < 8; attempt++) {
+            r = step_kernel_eager(kModeInit, true);
+            if (r) return r;
             Counters c;
             r = read_counters(&c);
             if (r) return r;
             r = check_fatal(c);
             if (r) return r;
-            if (!(c.error & kErrOverflow)) break;
+            if (!(c.error & kErrOverflow)) {
+                have_state = true;
+                return MD_OK;
+            }
             r = regrow(c);
             if (r) return r;
         }
-        r = step_kernel_eager(kModeInit, true);
-        if (r) return r;
-        Counters c;
-        r = read_counters(&c);
-        if (r) return r;
-        r = check_fatal(c);
-        if (r) return r;
-        have_state = true;
-        return MD_OK;
+        err = "neighbour list kept overflowing";
+        return MD_EOVERFLOW;
     }
 
     int step(int64_t n) override {
@@ -777,6 +796,14 @@ struct Sim : SimBase {
         if (!have_state) {
             err = "md_get_state before md_set_state";
             return MD_ESTATE;
+        }
+        if (device && direct(pos) && direct(vel)) {
+            Args<P> out = a;
+            out.io_pos = pos;
+            out.io_vel = vel;
+            MD_CUDA(launch(kt.get_state, grid_atoms(), kBlock, out));
+            MD_CUDA(cudaStreamSynchronize(stream));
+            return MD_OK;
         }
         MD_CUDA(launch(kt.get_state, grid_atoms(), kBlock, a));
         size_t bytes = sizeof(double) * 3 * (size_t)a.n;

@@ -198,13 +198,25 @@ __device__ __forceinline__ int wrap_add(int c, int d, int G) {
 // cell_of(md_get_state positions) equals the stored cells, element by
 // element, as the FP64 reference computes it.
 
+// (The FP64 pipe bounds the kernels that convert whole states, so what can be
+// had from integer operations is: c + 1/2 from the bits of 2^52 + c, whose
+// difference to 2^52 - 1/2 is exact, and the test below.)
 __device__ __forceinline__ double cell_centre(int c, double w, double hL) {
-    return __dsub_rn(__dmul_rn((double)c + 0.5, w), hL);
+    const double h = __dsub_rn(__hiloint2double(0x43300000, c), 4503599627370495.5);
+    return __dsub_rn(__dmul_rn(h, w), hL);
+}
+
+// Whether |x| is below hL by more than one part in 2^21 (the high words
+// differ): x then lies in [-L/2, L/2) and floor((x + L/2)/L) is 0, whatever
+// the rounding.  False for NaN and infinities.
+__device__ __forceinline__ bool surely_wrapped(double x, double hL) {
+    return (__double2hiint(x) & 0x7fffffff) < __double2hiint(hL);
 }
 
 template <class P>
 __device__ __forceinline__ double abs_coord(const Args<P>& a, int d, int c, double t) {
     const double x = __dadd_rn(cell_centre(c, a.w[d], a.hL[d]), t);
+    if (surely_wrapped(x, a.hL[d])) return x;
     const double s = floor(__dmul_rn(__dadd_rn(x, a.hL[d]), a.invL[d]));
     return __dsub_rn(x, __dmul_rn(s, a.L[d]));
 }
@@ -216,6 +228,11 @@ __device__ __forceinline__ double abs_coord(const Args<P>& a, int d, int c, doub
 // non-finite x and for a magnitude too large to have been wrapped.
 template <class P>
 __device__ __forceinline__ bool bin_coord(const Args<P>& a, int d, double x, int& c, double& t) {
+    if (surely_wrapped(x, a.hL[d])) {  // (x + L/2) G/L lies in [0, G): truncation is the floor
+        c = __double2int_rz(__dmul_rn(__dadd_rn(x, a.hL[d]), a.invW[d]));
+        t = __dsub_rn(x, cell_centre(c, a.w[d], a.hL[d]));
+        return true;
+    }
     if (!isfinite(x)) {
         c = 0;
         t = 0.0;
@@ -936,10 +953,12 @@ __device__ __forceinline__ void set_state_item(const Args<P>& a, int64_t i) {
     bool bad = false;
     for (int d = 0; d < 3; d++) {
         double x = a.io_pos[3 * i + d];
-        bad |= !isfinite(x);
-        if (!isfinite(x)) x = 0.0;
-        const double s = floor(__dmul_rn(__dadd_rn(x, a.hL[d]), a.invL[d]));
-        x = __dsub_rn(x, __dmul_rn(s, a.L[d]));
+        if (!surely_wrapped(x, a.hL[d])) {
+            bad |= !isfinite(x);
+            if (!isfinite(x)) x = 0.0;
+            const double s = floor(__dmul_rn(__dadd_rn(x, a.hL[d]), a.invL[d]));
+            x = __dsub_rn(x, __dmul_rn(s, a.L[d]));
+        }
         double t;
         bad |= !bin_coord(a, d, x, c[d], t);
         split_offset(t, pb[d], o[d]);

@@ -56,6 +56,46 @@ def test_cells_bit_exact(case, prec):
     s.close()
 
 
+@pytest.mark.parametrize("prec", PRECS)
+def test_loaded_positions_at_the_faces_and_far_outside(prec):
+    # coordinates where the wrap and the cell rule take their general path (at
+    # a face, one ulp beside it, several boxes away) beside ordinary ones: the
+    # cells are the reference's, and the load from device and from pinned host
+    # memory gives the same state
+    torch = pytest.importorskip("torch")
+    pos, vel, L = state(600, 0.3, 1.0, 61, aspect=(1.0, 1.3, 0.9))
+    h = 0.5 * np.asarray(L)
+    edge = []
+    for k in range(3):
+        for x in (-h[k], h[k], np.nextafter(h[k], 0.0), np.nextafter(-h[k], 0.0), np.nextafter(h[k], 9e9), 0.0, -0.0,
+                  h[k] * (1 - 2.0 ** -21), -h[k] * (1 - 2.0 ** -20), 7.25 * L[k], -1e6 * L[k]):
+            q = pos[len(edge)].copy()
+            q[k] = x
+            edge.append(q)
+    G = np.array(md.md_plan(L, 1, RC, 0.4, DT).G)
+    for q in edge:
+        one = md.Simulation(L, 1, RC, 0.4, DT, precision=prec)
+        zero = np.zeros((1, 3))
+        one.set_state(q[None], zero)
+        pw = oracle.wrap(q[None], L)
+        assert np.array_equal(one.cells(), oracle.cell_of(pw, L, G)), q
+        p1, _ = one.get_state()
+        # (one that rounds onto the upper face is reported as its image at the lower one)
+        assert np.abs(min_image(p1 - pw, L)).max() <= 4e-16 * np.max(L)
+        assert_same_cells(one.cells(), p1, L, G)
+        tq = torch.from_numpy(q[None].copy()).cuda()
+        tz = torch.zeros((1, 3), dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        one.set_state(tq, tz)
+        po, vo = torch.empty_like(tq), torch.empty_like(tz)
+        one.get_state(po, vo)
+        assert np.array_equal(po.cpu().numpy(), p1)
+        ph, vh = torch.empty((1, 3), dtype=torch.float64).pin_memory(), torch.empty((1, 3), dtype=torch.float64).pin_memory()
+        one.get_state(ph, vh)
+        assert np.array_equal(ph.numpy(), p1)
+        one.close()
+
+
 BUILDS = ["warp", "thread"]
 
 
