@@ -246,7 +246,10 @@ struct Sim : SimBase {
 
     unsigned grid_atoms() const { return (unsigned)a.nblocks; }
     static unsigned few(unsigned blocks) { return std::min(blocks, 8u * 152u); }  // eight blocks on an SM
-    unsigned grid_cells() const { return (unsigned)((a.ncells + kBlock - 1) / kBlock); }
+    unsigned grid_sort() const {
+        const int per = sort_cells(a.n, a.ncells);
+        return (unsigned)((a.ncells + per - 1) / per);
+    }
     unsigned grid_scatter() const {
         int64_t m = a.n > a.ncells ? a.n : a.ncells;
         return (unsigned)((m + kBlock - 1) / kBlock);
@@ -300,7 +303,7 @@ struct Sim : SimBase {
         MD_CUDA(launch(kt.bin, grid_atoms(), kBlock, a, g));
         MD_CUDA(launch(kt.scan_apply, (unsigned)a.ntiles, kBlock, a, g));
         MD_CUDA(launch(kt.scatter, grid_scatter(), kBlock, a, g));
-        MD_CUDA(launch(kt.sort_gather, few(grid_cells()), kBlock, a, g));
+        MD_CUDA(launch(kt.sort_gather, few(grid_sort()), kBlock, a, g));
         MD_CUDA(launch(kt.commit, few(grid_atoms()), kBlock, a, g));
         if (!prm.cell_list_only) MD_CUDA(launch(build_fn(), grid_build(), block_build(), a, g));
         MD_CUDA(launch(kt.rebuild_done, 1, 32, a, g));
@@ -372,7 +375,7 @@ struct Sim : SimBase {
         MD_CUDA(add(kt.bin, grid_atoms(), kBlock));
         MD_CUDA(add(kt.scan_apply, (unsigned)a.ntiles, kBlock));
         MD_CUDA(add(kt.scatter, grid_scatter(), kBlock));
-        MD_CUDA(add(kt.sort_gather, few(grid_cells()), kBlock));
+        MD_CUDA(add(kt.sort_gather, few(grid_sort()), kBlock));
         MD_CUDA(add(kt.commit, few(grid_atoms()), kBlock));
         if (!prm.cell_list_only) MD_CUDA(add(build_fn(), grid_build(), block_build()));
         MD_CUDA(add(kt.rebuild_done, 1, 32));
@@ -452,41 +455,51 @@ struct Sim : SimBase {
 
     int graph_kernels_per_step() const { return 1; }
 
-    // Whether plain steps run in the one-launch loop of md_run.cuh: the mixed
-    // form with sorted lists and the default kernels, and a system whose
-    // blocks are all resident at once (up to 29184 atoms).  It wins wherever
+    // Whether plain steps run in a one-launch loop of md_run.cuh: the
+    // cell-list-only variant, or the mixed form with sorted lists and the
+    // default kernels, and a system whose blocks are all resident at once
+    // (about 12000 and 29184 atoms).  It wins wherever
     // it applies: 100 steps and their read-back take 0.66 ms instead of 1.77
     // at 2048 atoms and 1.15 ms instead of 2.05 at 20011.
     bool use_run() {
-        if (P::kFp64 || prm.cell_list_only || !prm.shell_bins || prm.variant != 0 || warp_build() ||
-            use_direct_build(box, a.n, plan.rn))
-            return false;
-        const int block = run_block(a.n);
-        if (block == 0) return false;
+        if (run_threads() == 0) return false;
         if (run_blocks_max < 0) {
             int coop = 0, sms = 0, per_sm = 0;
             run_blocks_max = 0;
             if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess || !coop ||
                 cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, run_fn(block), block, 0) != cudaSuccess) {
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, run_fn(), run_threads(), 0) != cudaSuccess) {
                 cudaGetLastError();
                 return false;
             }
-            run_blocks_max = std::min(per_sm * sms, kRunMaxBlocks);
+            run_blocks_max = per_sm * sms;
         }
-        return run_grid(block) <= run_blocks_max;
+        return run_grid() <= run_blocks_max;
     }
-    void* run_fn(int block) const { return block == 128 ? kt.run_small : kt.run; }
-    int run_grid(int block) const { return (int)((a.n * kRunLanes + block - 1) / block); }
+    // threads per block of the loop's kernel (0: this system has none), its
+    // kernel and its blocks
+    int run_threads() const {
+        if (prm.cell_list_only) return kRunCellBlock;
+        if (P::kFp64 || !prm.shell_bins || prm.variant != 0 || warp_build() || use_direct_build(box, a.n, plan.rn))
+            return 0;
+        return run_block(a.n);
+    }
+    void* run_fn() const {
+        if (prm.cell_list_only) return kt.run_cells;
+        return run_threads() == 128 ? kt.run_small : kt.run;
+    }
+    int64_t run_grid() const {
+        const int64_t t = a.n * (prm.cell_list_only ? kCellLanes : kRunLanes);
+        return (t + run_threads() - 1) / run_threads();
+    }
 
     // Queues `count` plain steps as one-launch loops.
     int run_loop(int64_t count) {
-        const int block = run_block(a.n);
         while (count > 0) {
             long long k = std::min<int64_t>(count, kRunSteps);
             void* p[] = {(void*)&a, (void*)&k, (void*)&run_words};
             MD_CUDA(cudaMemsetAsync(run_words, 0, sizeof(unsigned long long) * 4 * kRunWordStride, stream));
-            MD_CUDA(cudaLaunchCooperativeKernel(run_fn(block), dim3(run_grid(block)), dim3(block), p, 0, stream));
+            MD_CUDA(cudaLaunchCooperativeKernel(run_fn(), dim3((unsigned)run_grid()), dim3(run_threads()), p, 0, stream));
             launches++;
             count -= k;
         }

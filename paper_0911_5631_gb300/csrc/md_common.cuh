@@ -86,6 +86,7 @@ constexpr int kRunMaxBlocks = 304;
 // before a wait is given up (at half a microsecond or more each).
 constexpr int kRunSteps = 2048;
 constexpr int kRunPolls = 1 << 21;
+constexpr int kRunCellBlock = 128;  // threads per block of the cell-list-only loop
 constexpr int kRunWordStride = 16;  // 64-bit words between the barrier's four words
 // Elements per block of the cell-count scan (kBlock threads x 8).
 constexpr int kScanTile = 2048;
@@ -268,6 +269,12 @@ __host__ __device__ __forceinline__ int64_t pair_slots(int64_t n) {
     int64_t s = 1;
     while (s < n) s <<= 1;
     return s;
+}
+
+// Cells of a block of k_sort_gather.
+__host__ __device__ __forceinline__ int sort_cells(int64_t n, int64_t ncells) {
+    const int64_t per_cell = n / ncells > 1 ? n / ncells : 1;
+    return per_cell < kBlock / 8 ? (int)(kBlock / per_cell) : 8;
 }
 
 // Entry m of atom i's neighbour list (Sec. 3.4, W_{m,i}) sits at

@@ -810,28 +810,27 @@ __device__ __forceinline__ void forces_mixed(const Args<Mixed>& a, int cnt, cons
 //
 // Mixed form: the copy holds the pair coordinates themselves and the lanes'
 // integer sums add up to the same bits in any split.
+constexpr int kCellQueue = 16;  // survivors an atom queues (FP64 form)
+// The forces on the atom in slot s (in = false: none), in all of its lanes;
+// returns the atom.  pc: the current pair coordinates; queue: the atom's
+// kCellQueue ints (FP64 form).  Every lane of the warp must call it.
 template <class P, bool kEnergy>
-__global__ void __launch_bounds__(kBlock) k_cell_forces(Args<P> a) {
+__device__ __forceinline__ int cell_forces_item(const Args<P>& a, int64_t s, bool in,
+                                                const typename P::pos4* pc, int* queue,
+                                                typename AccOf<P>::type& acc) {
     using real = typename P::real;
-    using Acc = typename AccOf<P>::type;
     constexpr unsigned kFull = 0xffffffffu;
-    constexpr int kQueue = 16;   // survivors an atom queues (FP64 form)
+    constexpr int kQueue = kCellQueue;
     constexpr int kCells = (27 + kCellLanes - 1) / kCellLanes;  // cells of a lane
     constexpr int kFirst = 2;    // candidates of a cell loaded ahead (a cell holds about one)
     static_assert(kCellLanes == 8, "the queue's bookkeeping");
-    __shared__ int s_queue[P::kFp64 ? kBlock / kCellLanes * kQueue : 1];
     const int lane = threadIdx.x & 31, sub = lane % kCellLanes, shift = lane - sub;
     const unsigned below = (1u << sub) - 1u;
-    const int64_t s = gtid() / kCellLanes;
-    const bool in = s < a.n;
     const float4 ci = a.cand[in ? s : 0];
     const int i = __float_as_int(ci.w);
     int cx, cy, cz;
     unpack_cell(a.cell[i], cx, cy, cz);
-    const typename P::pos4* pc = a.ctr->parity ? a.pB : a.pA;
-    const typename P::pos4 qi = ld_pos4(pc + i);
-    int* queue = s_queue + (P::kFp64 ? (int)(threadIdx.x / kCellLanes) * kQueue : 0);
-    Acc acc;
+    const typename P::pos4 qi = pc[i];
     int nq = 0;
 
     auto evaluate = [&]() {  // (FP64 form) the queued pairs, one a lane
@@ -839,7 +838,7 @@ __global__ void __launch_bounds__(kBlock) k_cell_forces(Args<P> a) {
         for (int p = sub; __any_sync(kFull, p < nq); p += kCellLanes) {
             if (p >= nq) continue;
             const unsigned e = (unsigned)queue[p];
-            const auto pj = ld_pos4(pc + (e & a.jmask));
+            const typename P::pos4 pj = pc[e & a.jmask];
             const unsigned c = e >> kCodeShift;
             const real dx = (qi.x - pj.x) + (real)(1 - (int)(c & 3u)) * (real)a.w[0];
             const real dy = (qi.y - pj.y) + (real)(1 - (int)((c >> 2) & 3u)) * (real)a.w[1];
@@ -885,14 +884,14 @@ __global__ void __launch_bounds__(kBlock) k_cell_forces(Args<P> a) {
     for (int q = 0; q < kCells; q++)
 #pragma unroll
         for (int u = 0; u < kFirst; u++)
-            first[q][u] = lo[q] + u < hi[q] ? __ldg(a.cand + lo[q] + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+            first[q][u] = lo[q] + u < hi[q] ? a.cand[lo[q] + u] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int q = 0; q < kCells; q++) {
         const int d = sub + kCellLanes * q;
 #pragma unroll
         for (int u = 0; u < kFirst; u++) test(first[q][u], lo[q] + u < hi[q], d);
         for (int t = lo[q] + kFirst; __any_sync(kFull, t < hi[q]); t++)
-            test(t < hi[q] ? __ldg(a.cand + t) : make_float4(0.f, 0.f, 0.f, 0.f), t < hi[q], d);
+            test(t < hi[q] ? a.cand[t] : make_float4(0.f, 0.f, 0.f, 0.f), t < hi[q], d);
     }
     if constexpr (P::kFp64) evaluate();
 
@@ -925,6 +924,19 @@ __global__ void __launch_bounds__(kBlock) k_cell_forces(Args<P> a) {
             total(acc.w);
         }
     }
+    return i;
+}
+
+template <class P, bool kEnergy>
+__global__ void __launch_bounds__(kBlock) k_cell_forces(Args<P> a) {
+    __shared__ int s_queue[P::kFp64 ? kBlock / kCellLanes * kCellQueue : 1];
+    const int lane = threadIdx.x & 31, sub = lane % kCellLanes;
+    const int64_t s = gtid() / kCellLanes;
+    const bool in = s < a.n;
+    typename AccOf<P>::type acc;
+    const int i = cell_forces_item<P, kEnergy>(a, s, in, a.ctr->parity ? a.pB : a.pA,
+                                               s_queue + (P::kFp64 ? (int)(threadIdx.x / kCellLanes) * kCellQueue : 0),
+                                               acc);
     if (in && sub == 0) {
         a.fx[i] = acc.force_x();
         a.fy[i] = acc.force_y();
@@ -934,7 +946,7 @@ __global__ void __launch_bounds__(kBlock) k_cell_forces(Args<P> a) {
             a.s_oy[i] = 0.5 * acc.virial();
         }
     }
-    if (__any_sync(kFull, in && acc.close) && lane == 0) atomicOr(&a.ctr->close_flag, 1);
+    if (__any_sync(0xffffffffu, in && acc.close) && lane == 0) atomicOr(&a.ctr->close_flag, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -1078,9 +1090,13 @@ __device__ __forceinline__ int bin_item(const Args<P>& a, int64_t i, int parity)
     typename P::pos4* pc = parity ? a.pB : a.pA;
     const real p0 = pair_coord(pb[0], o[0]), p1 = pair_coord(pb[1], o[1]), p2 = pair_coord(pb[2], o[2]);
     pc[i] = make_pos4(p0, p1, p2, pair_payload(a, pack_cell(cc[0], cc[1], cc[2]), p0, p1, p2));
-    const int c = cell_index(cc[0], cc[1], cc[2], a.G);
+    return cell_index(cc[0], cc[1], cc[2], a.G);
+}
+
+// Counts atom i in its cell c; its rank is the order of arrival.
+template <class P>
+__device__ __forceinline__ void count_item(const Args<P>& a, int64_t i, int c) {
     a.rank[i] = atomicAdd(&a.count[c], 1);
-    return c;
 }
 
 // Binning of every atom, and phase 1 of the exclusive scan of the cell
@@ -1097,7 +1113,12 @@ __global__ void __launch_bounds__(kBlock) k_bin(Args<P> a, int guard) {
         C->list_entries = 0;
     }
     const int64_t i = gtid();
-    const int tile = i < a.n ? bin_item<P>(a, i, C->parity) / kScanTile : -1;
+    int tile = -1;
+    if (i < a.n) {
+        const int c = bin_item<P>(a, i, C->parity);
+        count_item<P>(a, i, c);
+        tile = c / kScanTile;
+    }
     const unsigned peers = __match_any_sync(0xffffffffu, tile);
     if (tile >= 0 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&a.tile_sum[tile], __popc(peers));
 }
@@ -1241,19 +1262,24 @@ __device__ __forceinline__ void gather_item(const Args<P>& a, int64_t s, int reo
     }
 }
 
-// Sorts and gathers each cell, a thread per cell.  Most rebuilds of the mixed
-// form have neither to do, and 4096 blocks that return at once take 5 us, so
-// this kernel and k_commit run few blocks that stride.
+// Sorts each cell, a thread per cell, and gathers the cells' slots, a thread
+// per slot; a block takes about as many cells as hold its threads' number of
+// slots.  Most rebuilds of the mixed form have neither to do, and 4096 blocks
+// that return at once take 5 us, so this kernel and k_commit run few blocks
+// that stride.
 template <class P>
 __global__ void __launch_bounds__(kBlock) k_sort_gather(Args<P> a, int guard) {
     const Counters* C = a.ctr;
     if (guard && !C->rebuild_flag) return;
     const int reorder = C->reorder_now;
     if (!sorts_cells<P>(reorder)) return;
-    for (int64_t c = gtid(); c < a.ncells; c += (int64_t)gridDim.x * blockDim.x) {
-        cellsort_item<P>(a, c);
-        const int end = min(a.cell_start[c + 1], (int)a.n);
-        for (int s = a.cell_start[c]; s < end; s++) gather_item<P>(a, s, reorder);
+    const int per = sort_cells(a.n, a.ncells);
+    for (int64_t c0 = (int64_t)blockIdx.x * per; c0 < a.ncells; c0 += (int64_t)gridDim.x * per) {
+        const int64_t c1 = min(c0 + per, (int64_t)a.ncells);
+        if (c0 + threadIdx.x < c1) cellsort_item<P>(a, c0 + threadIdx.x);
+        __syncthreads();  // the block's cells are in order
+        const int end = min(a.cell_start[c1], (int)a.n);
+        for (int s = a.cell_start[c0] + (int)threadIdx.x; s < end; s += kBlock) gather_item<P>(a, s, reorder);
     }
 }
 
@@ -2524,7 +2550,7 @@ template <class P>
 __device__ __noinline__ void ens_rebuild(const Args<P>& a, EnsShared& sh, int* stage, Team tm) {
     Counters* C = a.ctr;
     const int64_t n = a.n, t0 = tm.first(), dt = tm.stride();
-    for (int64_t i = t0; i < n; i += dt) bin_item<P>(a, i, C->parity);
+    for (int64_t i = t0; i < n; i += dt) count_item<P>(a, i, bin_item<P>(a, i, C->parity));
     tm.sync();
     if (tm.lead_block()) ens_scan<P>(a, sh);
     tm.sync();
@@ -2831,6 +2857,7 @@ KernelTable<P> make_kernel_table() {
     t.rescale = (void*)k_rescale<P>;
     t.count_reads = (void*)k_count_reads<P>;
     t.spin = (void*)k_spin<P>;
+    t.run_cells = (void*)k_run_cells<P>;
     if constexpr (!P::kFp64) {
         t.ensemble = (void*)k_ensemble<P>;
         t.run_small = (void*)k_run<P, 128>;

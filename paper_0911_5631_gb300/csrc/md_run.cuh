@@ -11,7 +11,11 @@
 // barrier.  The mixed form's force sums are integers, so the trajectory is
 // the one of the step kernels, bit for bit.
 //
-// Included by md_kernels.cuh; mixed form with a neighbour list only.
+// k_run_cells does the same for the cell-list-only variant, in both forms: its
+// rebuild at every step leaves nothing to keep in registers, but saves the ten
+// launches of a step.
+//
+// Included by md_kernels.cuh.
 #pragma once
 
 namespace md {
@@ -313,7 +317,12 @@ __device__ __noinline__ int run_rebuild(const Args<P>& a, int64_t i, int par, in
         C->list_entries = 0;
     }
     if (blockIdx.x == 0 && threadIdx.x < kD2Buckets) a.d2b[threadIdx.x * 32] = 0u;  // displacements count from here
-    const int tile = in && sub == 0 ? bin_item<P>(a, i, par) / kScanTile : -1;
+    int tile = -1;
+    if (in && sub == 0) {
+        const int c = bin_item<P>(a, i, par);
+        count_item<P>(a, i, c);
+        tile = c / kScanTile;
+    }
     const unsigned peers = __match_any_sync(kFull, tile);
     if (tile >= 0 && lane == __ffs(peers) - 1) atomicAdd(&a.tile_sum[tile], __popc(peers));
     int said = bar.sync(0, s_sync, C);
@@ -518,6 +527,104 @@ __global__ void __launch_bounds__(kB, kB == kRunMaxBlock ? 2 : 1) k_run(Args<P> 
         C->reorders += reorders;
         C->far_flag = 0u;
         C->reach = kShellBins;  // the next step reads every entry; its closing kernel sets the reach again
+    }
+}
+
+// Up to `steps` plain steps of the cell-list-only variant, kCellLanes lanes
+// per atom in the force phase.  The phases of a step are the kernels of the
+// graph, a grid barrier between them, with the same operations in the same
+// order, so the results are the same bits.  Cooperative launch of
+// ceil(n kCellLanes / kRunCellBlock) blocks.
+template <class P>
+__global__ void __launch_bounds__(kRunCellBlock, 5) k_run_cells(Args<P> a, long long steps, unsigned long long* words) {
+    using real = typename P::real;
+    __shared__ int s_queue[P::kFp64 ? kRunCellBlock / kCellLanes * kCellQueue : 1];
+    __shared__ int s_sync;
+    __shared__ int s_scan[32];
+    Counters* C = a.ctr;
+    RunBarrier bar{words, 0u};
+    const int sub = threadIdx.x % kCellLanes;
+    const int64_t slot = ((int64_t)blockIdx.x * kRunCellBlock + threadIdx.x) / kCellLanes;
+    const int64_t t0 = (int64_t)blockIdx.x * kRunCellBlock + threadIdx.x, dt = (int64_t)gridDim.x * kRunCellBlock;
+    int* queue = s_queue + (P::kFp64 ? (int)(threadIdx.x / kCellLanes) * kCellQueue : 0);
+    const int err0 = C->error;
+    int par = C->parity, reorder = C->reorder_now;
+    const int todo = (int)min(steps, C->steps_left - 1);  // (steps is at most kRunSteps)
+    int since = (int)min(C->since_reorder, (long long)INT_MAX / 2);
+    if (err0 != 0 || todo <= 0) return;
+    int reorders = 0, done = 0, stop = 0;
+    while (done < todo && !stop) {
+        // the rebuild (k_bin .. k_rebuild_done); the grid has a thread for
+        // every atom several times over: the first n of them take one each
+        if (t0 == 0) C->max_occ = 0;
+        int tile = -1;
+        if (t0 < a.n) {
+            const int c = bin_item<P>(a, t0, par);
+            count_item<P>(a, t0, c);
+            tile = c / kScanTile;
+        }
+        const unsigned peers = __match_any_sync(0xffffffffu, tile);
+        if (tile >= 0 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&a.tile_sum[tile], __popc(peers));
+        bar.sync(0, &s_sync, C);
+        for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) run_scan_tile(a, t, s_scan);
+        bar.sync(0, &s_sync, C);
+        if (t0 < a.n) scatter_item<P>(a, t0, reorder);
+        for (int64_t c = t0; c < a.ncells; c += dt) a.count[c] = 0;
+        for (int64_t c = t0; c < a.ntiles; c += dt) a.tile_sum[c] = 0;
+        bar.sync(0, &s_sync, C);
+        if (sorts_cells<P>(reorder)) {
+            for (int64_t c = t0; c < a.ncells; c += dt) {
+                cellsort_item<P>(a, c);
+                const int end = min(a.cell_start[c + 1], (int)a.n);
+                for (int s = a.cell_start[c]; s < end; s++) gather_item<P>(a, s, reorder);
+            }
+            bar.sync(0, &s_sync, C);
+            if (reorder) {
+                if (t0 < a.n) commit_item<P>(a, t0, par);
+                bar.sync(0, &s_sync, C);
+                reorders++;
+                since = 0;
+            }
+        }
+        // forces, and the step's update of one component in each of three lanes
+        const typename P::pos4* pc = par ? a.pB : a.pA;
+        typename P::pos4* pn = par ? a.pA : a.pB;
+        typename AccOf<P>::type acc;
+        const bool in = slot < a.n;
+        const int i = cell_forces_item<P, false>(a, slot, in, pc, queue, acc);
+        if (in && sub < 3) {
+            typename P::vel* vp = sub == 0 ? a.vx : (sub == 1 ? a.vy : a.vz);
+            double* op = sub == 0 ? a.ox : (sub == 1 ? a.oy : a.oz);
+            const real f = sub == 0 ? acc.force_x() : (sub == 1 ? acc.force_y() : acc.force_z());
+            const real pb = (sub == 0 ? a.pbx : (sub == 1 ? a.pby : a.pbz))[i];
+            const typename P::vel v = kick(a, kick(a, vp[i], f), f);
+            const double o = drift(op[i], v, a.dt);
+            real p;
+            moved<true>(pb, o, p);
+            vp[i] = v;
+            op[i] = o;
+            reinterpret_cast<real*>(pn + i)[sub] = p;
+        }
+        if (in && acc.close) atomicOr(&C->error, kErrClose);
+        stop = bar.sync((in && acc.close) || __ldcg(&C->error) != 0 ? kRunStop : 0, &s_sync, C) & kRunStop;
+        par ^= 1;
+        done++;
+        since++;
+        reorder = a.reorder_interval > 0 && since >= a.reorder_interval;
+    }
+    if (t0 == 0) {  // (no block reads the counters any more)
+        C->parity = par;
+        C->rebuild_flag = 1;  // as after every step of this variant
+        C->reorder_now = reorder;
+        C->steps_left -= done;
+        C->step += done;
+        C->since_reorder = reorders > 0 ? since : C->since_reorder + done;
+        C->rebuilds += done;
+        C->run_rebuilds += done;
+        C->reorders += reorders;
+        C->far_flag = 0u;
+        C->max_nn = 0;
+        C->list_entries = 0;
     }
 }
 

@@ -39,6 +39,7 @@ struct KernelTable {
     void* count_reads;
     void* spin;
     void* ensemble;  // mixed form only (nullptr for FP64)
+    void* run_cells;  // the one-launch step loop of small cells-only systems
     void* run_small;  // the one-launch step loop of small systems, blocks of 128 threads
     void* run;       // the one-launch step loop of small systems, mixed form only
     // step-kernel variants of the paper's ablations, mixed list form only

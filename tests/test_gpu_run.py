@@ -65,3 +65,27 @@ def test_run_loop_grows_its_lists_and_reports_errors():
     p, v = s.get_state()
     s.close()
     assert np.array_equal(p, b[0]) and np.array_equal(v, b[1])
+
+
+# the cell-list-only loop (8 lanes per atom, 16 atoms per block; the last size
+# is beyond the resident blocks and runs as graphs), both forms
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("n,rho,T,reorder", [(17, 0.2, 1.0, 100), (500, 0.8, 1.0, 7), (2049, 1.0, 2.0, 20),
+                                             (9000, 0.7, 1.0, 0), (30000, 0.8, 1.0, 25)])
+def test_cells_only_loop_matches_stream_launches(n, rho, T, reorder, prec):
+    pos, vel, L = state(n, rho, T, 53, jitter=0.05)
+    steps = [1, 2, 40, 23]
+    out = []
+    for graphs in (True, False):
+        s = md.Simulation(L, n, RC, 0.0, DT, precision=prec, cell_list_only=True, reorder_interval=reorder,
+                          use_graphs=graphs)
+        s.set_state(pos, vel)
+        for k in steps:
+            s.step(k)
+        out.append(s.get_state() + (s.measure(), s.cells()))
+        s.close()
+    a, b = out
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1]) and np.array_equal(a[3], b[3])
+    for k in ("step", "rebuilds", "reorders", "max_occupancy", "ke", "pe", "virial"):
+        assert a[2][k] == b[2][k], k
+    assert a[2]["rebuilds"] == 1 + sum(steps)
