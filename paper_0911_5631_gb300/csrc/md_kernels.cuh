@@ -532,6 +532,78 @@ struct AccMixed {
     __device__ __forceinline__ void force(const Args<Mixed>& a, float dx, float dy, float dz, float r2) {
         force<kEnergy>(a, f2(dx, dy), dz, r2);
     }
+    // Two entries of a list at once, an entry in each half of a packed pair:
+    // separations (dx, dy, dz), in0 / in1 say which of the two is an entry at
+    // all.  Every operation is the one force() does on each half, in its
+    // order, so the sums get the same integers; an entry that does not
+    // interact gets f/r = 0 and adds nothing.  No branch but the rare one of
+    // a large force: a warp would take a branch per entry for any of its 32
+    // atoms anyway.  The raw bit patterns are summed, and `raw` counts the
+    // terms whose kFixMagicBits are still to be taken out (settle).
+    int raw = 0;
+    __device__ __forceinline__ static void add_small2(Fix& f, F2 g) {
+        const F2 M = f2(kFixMagic, kFixMagic);
+        float lo, hi;
+        const F2 s2 = f2_fma(g, f2(1024.0f, 1024.0f), M);
+        f2_get(s2, lo, hi);
+        f.b = (int)((unsigned)f.b + __float_as_uint(lo) + __float_as_uint(hi));
+        const F2 r2 = f2_fma(f2_sub(s2, M), f2(-0x1p-10f, -0x1p-10f), g);
+        const F2 s3 = f2_fma(r2, f2(4294967296.0f, 4294967296.0f), M);
+        f2_get(s3, lo, hi);
+        f.c = (int)((unsigned)f.c + __float_as_uint(lo) + __float_as_uint(hi));
+    }
+    __device__ __forceinline__ void force2(const Args<Mixed>& a, F2 dx, F2 dy, F2 dz, bool in0, bool in1) {
+        // (dx^2 + dy^2 by scalar additions: a packed product and sum would be
+        // fused into one rounding)
+        float x0, x1, y0, y1, r0, r1;
+        f2_get(f2_mul(dx, dx), x0, x1);
+        f2_get(f2_mul(dy, dy), y0, y1);
+        const F2 rr = f2_fma(dz, dz, f2(__fadd_rn(x0, y0), __fadd_rn(x1, y1)));
+        f2_get(rr, r0, r1);
+        const F2 ir2 = f2(__fdividef(1.0f, r0), __fdividef(1.0f, r1));
+        const F2 ir6 = f2_mul(f2_mul(ir2, ir2), ir2);
+        const F2 fr = f2_mul(f2_mul(f2_mul(f2(48.0f, 48.0f), ir6), f2_sub(ir6, f2(0.5f, 0.5f))), ir2);
+        float f0, f1;
+        f2_get(fr, f0, f1);
+        f0 = in0 && r0 < a.rc2f ? f0 : 0.0f;
+        f1 = in1 && r1 < a.rc2f ? f1 : 0.0f;
+        if (!(fmaxf(f0, f1) < a.fix_small_fr)) {  // (f/r = inf, from r = 0, among them)
+            if (!(f0 < a.fix_small_fr)) {
+                large(a, dx, dy, dz, f0, r0, false);
+                f0 = 0.0f;
+            }
+            if (!(f1 < a.fix_small_fr)) {
+                large(a, dx, dy, dz, f1, r1, true);
+                f1 = 0.0f;
+            }
+        }
+        const F2 f = f2(f0, f1);
+        add_small2(fxy.x, f2_mul(f, dx));
+        add_small2(fxy.y, f2_mul(f, dy));
+        add_small2(fz, f2_mul(f, dz));
+        raw += 2;
+    }
+    __device__ __forceinline__ void large(const Args<Mixed>& a, F2 dx, F2 dy, F2 dz, float fr, float r2, bool second) {
+        float x0, x1, y0, y1, z0, z1;
+        f2_get(dx, x0, x1);
+        f2_get(dy, y0, y1);
+        f2_get(dz, z0, z1);
+        close |= (r2 < a.close2f);
+        fxy.x.add(fr * (second ? x1 : x0));
+        fxy.y.add(fr * (second ? y1 : y0));
+        fz.add(fr * (second ? z1 : z0));
+    }
+    __device__ __forceinline__ void settle() {
+        const unsigned k = (unsigned)raw * (unsigned)kFixMagicBits;  // (modulo 2^32, as the sums)
+        auto less = [&](int& x) { x = (int)((unsigned)x - k); };
+        less(fxy.x.b);
+        less(fxy.x.c);
+        less(fxy.y.b);
+        less(fxy.y.c);
+        less(fz.b);
+        less(fz.c);
+        raw = 0;
+    }
     __device__ __forceinline__ float r2(float dx, float dy, float dz) const { return fmaf(dx, dx, fmaf(dy, dy, dz * dz)); }
     __device__ __forceinline__ bool inside(const Args<Mixed>& a, float r2) const { return r2 < a.rc2f; }
     template <bool kEnergy>
@@ -719,13 +791,17 @@ __device__ __forceinline__ void forces_fp64(const Args<F64>& a, int cnt, const i
     if (__any_sync(kFull, nq > 0)) flush();
 }
 
-// Mixed-form counterpart of forces_fp64, in one pass: each entry's pair
-// term is evaluated as soon as its distance test passes.  Here a
-// shared-memory queue and a shift table cost more L1 data-pipe
-// wavefronts than the divergence they save, so the shift
+// Mixed-form counterpart of forces_fp64, in one pass: entries are evaluated
+// two at a time as they are gathered, in packed operations without a branch
+// (AccMixed::force2).  Here a shared-memory queue and a shift table cost more
+// L1 data-pipe wavefronts than the divergence they save, so the shift
 // -d w = (1 - k) w of each component (k the 2-bit code) is computed from
 // the code, and the staged rows and the rest of the column run as two loops
-// (no per-entry choice of source).  x and y travel as one packed pair.
+// (no per-entry choice of source).  What bounds it is the issue of these
+// instructions and the latency of the gathers.  An entry at a time, its pair
+// term behind a branch, took 267 us per step for 1M Lennard-Jones atoms (87
+// entries, half of them interacting) against 245 now, and 39.4 against 38.6
+// for 1M soft spheres right after a rebuild.
 __device__ __forceinline__ float small_int_to_float(unsigned k) {  // exact for k < 2^22
     return __uint_as_float(0x4B400000u | k) - 12582912.0f;
 }
@@ -744,28 +820,57 @@ __device__ __forceinline__ float4 gather4(const float4* p) {
     }
 }
 
+// Two entries e0, e1 (in1: e1 is one) whose pair coordinates are p0, p1.  Each
+// component of the two travels as a packed pair, from the cell codes on: the
+// code fields are masked in place and scaled by w, w/4 and w/16, so that the
+// shift (1 - k) w is exact.
+__device__ __forceinline__ void mixed_pair2(const Args<Mixed>& a, float qx, float qy, float qz, unsigned e0,
+                                            const float4& p0, unsigned e1, const float4& p1, bool in1, AccMixed& acc) {
+    const unsigned c0 = e0 >> kCodeShift, c1 = e1 >> kCodeShift;
+    auto field = [](unsigned x, unsigned y) {  // two small integers as floats
+        return f2_sub(f2(__uint_as_float(0x4B400000u | x), __uint_as_float(0x4B400000u | y)),
+                      f2(12582912.0f, 12582912.0f));
+    };
+    const float wx = a.wf[0], wy = a.wf[1], wz = a.wf[2];
+    const F2 sx = f2_fma(field(c0 & 3u, c1 & 3u), f2(-wx, -wx), f2(wx, wx));
+    const F2 sy = f2_fma(field(c0 & 12u, c1 & 12u), f2(-0.25f * wy, -0.25f * wy), f2(wy, wy));
+    const F2 sz = f2_fma(field(c0 & 48u, c1 & 48u), f2(-0.0625f * wz, -0.0625f * wz), f2(wz, wz));
+    const F2 dx = f2_add(f2_sub(f2(qx, qx), f2(p0.x, p1.x)), sx);
+    const F2 dy = f2_add(f2_sub(f2(qy, qy), f2(p0.y, p1.y)), sy);
+    const F2 dz = f2_add(f2_sub(f2(qz, qz), f2(p0.z, p1.z)), sz);
+    acc.force2(a, dx, dy, dz, true, in1);
+}
+
 template <bool kEnergy, bool kLdg = true, bool kRows = false>
 __device__ __forceinline__ void forces_mixed(const Args<Mixed>& a, int cnt, const int* col, const int* rows,
                                              int staged, float qx, float qy, float qz,
                                              const float4* __restrict__ pc, AccMixed& acc) {
     const unsigned jmask = a.jmask;  // entries are always < n; the mask only guards memory
     const int lane = threadIdx.x & 31;
-    const F2 qxy = f2(qx, qy);
-    const F2 wxy = f2(a.wf[0], a.wf[1]);
-    const F2 nwxy = f2(-a.wf[0], -a.wf[1]);
-    const float wz = a.wf[2];
     const float rc2 = a.rc2f;
+    // one entry, for the final step's energies
     auto pair = [&](unsigned e, const float4& pj) {
         const unsigned c = e >> kCodeShift;
         const F2 kxy = f2(small_int_to_float(c & 3u), small_int_to_float((c >> 2) & 3u));
-        const F2 sxy = f2_fma(kxy, nwxy, wxy);  // (1 - k) w, exact
-        const float sz = fmaf(small_int_to_float(c >> 4), -wz, wz);
-        const F2 dxy = f2_add(f2_sub(qxy, f2(pj.x, pj.y)), sxy);
+        const F2 sxy = f2_fma(kxy, f2(-a.wf[0], -a.wf[1]), f2(a.wf[0], a.wf[1]));  // (1 - k) w, exact
+        const float sz = fmaf(small_int_to_float(c >> 4), -a.wf[2], a.wf[2]);
+        const F2 dxy = f2_add(f2_sub(f2(qx, qy), f2(pj.x, pj.y)), sxy);
         const float dz = (qz - pj.z) + sz;
         float sx, sy;
         f2_get(f2_mul(dxy, dxy), sx, sy);
         const float rr = fmaf(dz, dz, sx + sy);
         if (rr < rc2) acc.template force<kEnergy>(a, dxy, dz, rr);
+    };
+    auto four = [&](const unsigned (&e)[4], const float4 (&pj)[4], int left) {  // left: entries there are
+        if constexpr (kEnergy) {
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (k < left) pair(e[k], pj[k]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; k += 2)
+                if (k < left) mixed_pair2(a, qx, qy, qz, e[k], pj[k], e[k + 1], pj[k + 1], k + 1 < left, acc);
+        }
     };
     const int ns = min(cnt, staged);  // staged is a multiple of 4 or the capacity
     int m = 0;
@@ -776,10 +881,8 @@ __device__ __forceinline__ void forces_mixed(const Args<Mixed>& a, int cnt, cons
         for (int k = 0; k < 4; k++) e[k] = (unsigned)rows[(m + k) * 32 + lane];  // rows past ns are unused
 #pragma unroll
         for (int k = 0; k < 4; k++)
-            if (m + k < ns) pj[k] = gather4<kLdg>(pc + (e[k] & jmask));
-#pragma unroll
-        for (int k = 0; k < 4; k++)
-            if (m + k < ns) pair(e[k], pj[k]);
+            pj[k] = m + k < ns ? gather4<kLdg>(pc + (e[k] & jmask)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        four(e, pj, ns - m);
     }
     constexpr int kStride = kRows ? 1 : 32;
     for (m = ns; m < cnt; m += 4) {
@@ -789,11 +892,10 @@ __device__ __forceinline__ void forces_mixed(const Args<Mixed>& a, int cnt, cons
         for (int k = 0; k < 4; k++) e[k] = (m + k < cnt) ? (unsigned)__ldcs(col + (size_t)(m + k) * kStride) : 0u;
 #pragma unroll
         for (int k = 0; k < 4; k++)
-            if (m + k < cnt) pj[k] = gather4<kLdg>(pc + (e[k] & jmask));
-#pragma unroll
-        for (int k = 0; k < 4; k++)
-            if (m + k < cnt) pair(e[k], pj[k]);
+            pj[k] = m + k < cnt ? gather4<kLdg>(pc + (e[k] & jmask)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        four(e, pj, cnt - m);
     }
+    if constexpr (!kEnergy) acc.settle();
 }
 
 // Forces straight from the 27 cells around each atom's cell (cell-list-only
@@ -1946,7 +2048,7 @@ __device__ __forceinline__ bool kickdrift_item(const Args<P>& a, int64_t i, type
     pc[i] = make_pos4(px, py, pz, pair_payload(a, P::kFp64 ? a.cell[i] : 0, px, py, pz));
     d2b = d2_bits(d2);
     if constexpr (P::kFp64) return d2 >= a.thr2;
-    else return d2 >= a.thr2f;
+    else return !(d2 < a.thr2f);
 }
 
 // First half of the first step of an md_step call (Sec. 3.1 (a)): half kick
@@ -2100,7 +2202,7 @@ __device__ __forceinline__ void step_atom(const Args<P>& a, int64_t i, bool in, 
             pn[i] = make_pos4(px, py, pz, pair_payload(a, P::kFp64 && !kCells ? a.cell[i] : 0, px, py, pz));
             d2b = d2_bits(d2);
             if constexpr (P::kFp64) far = d2 >= a.thr2;
-            else far = d2 >= a.thr2f;
+            else far = !(d2 < a.thr2f);  // (a NaN asks for the rebuild, which reports it)
         }
     }
 }

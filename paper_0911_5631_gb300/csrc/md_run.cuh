@@ -22,6 +22,7 @@ namespace md {
 
 constexpr int kRunRegs = 4;    // entries a lane keeps in registers: 16 per atom (12 in a fluid's list)
 constexpr int kRunStage = 10;  // candidates a lane of the build stages (an atom's four lanes: 40)
+static_assert(kRunRegs % 2 == 0, "entries are evaluated in pairs");
 static_assert(kRunLanes * kRunStage < 256, "one byte per shell bin in a 64-bit word");
 
 // What the blocks tell one another at a barrier.
@@ -443,29 +444,20 @@ __global__ void __launch_bounds__(kB, kB == kRunMaxBlock ? 2 : 1) k_run(Args<P> 
         float4 pj[kRunRegs];
 #pragma unroll
         for (int k = 0; k < kRunRegs; k++)
-            if (sub + kRunLanes * k < nn) pj[k] = gather4<false>(pc + (e[k] & a.jmask));
-        const F2 qxy = f2(__shfl_sync(kFull, p, lead), __shfl_sync(kFull, p, lead + 1));
-        const float qz = __shfl_sync(kFull, p, lead + 2);
+            pj[k] = sub + kRunLanes * k < nn ? gather4<false>(pc + (e[k] & a.jmask)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float qx = __shfl_sync(kFull, p, lead), qy = __shfl_sync(kFull, p, lead + 1),
+                    qz = __shfl_sync(kFull, p, lead + 2);
         AccMixed acc;
-        auto pair = [&](const float4& q, unsigned x) {  // the pair of forces_mixed
-            const unsigned c = x >> kCodeShift;
-            const F2 kxy = f2(small_int_to_float(c & 3u), small_int_to_float((c >> 2) & 3u));
-            const F2 hxy = f2_fma(kxy, f2(-a.wf[0], -a.wf[1]), f2(a.wf[0], a.wf[1]));  // (1 - k) w, exact
-            const float hz = fmaf(small_int_to_float(c >> 4), -a.wf[2], a.wf[2]);
-            const F2 dxy = f2_add(f2_sub(qxy, f2(q.x, q.y)), hxy);
-            const float dz = (qz - q.z) + hz;
-            float sx, sy;
-            f2_get(f2_mul(dxy, dxy), sx, sy);
-            const float rr = fmaf(dz, dz, sx + sy);
-            if (rr < a.rc2f) acc.template force<false>(a, dxy, dz, rr);
-        };
 #pragma unroll
-        for (int k = 0; k < kRunRegs; k++)
-            if (sub + kRunLanes * k < nn) pair(pj[k], e[k]);
+        for (int k = 0; k < kRunRegs; k += 2)
+            if (sub + kRunLanes * k < nn)
+                mixed_pair2(a, qx, qy, qz, e[k], pj[k], e[k + 1], pj[k + 1], sub + kRunLanes * (k + 1) < nn, acc);
         for (int m = sub + kRunLanes * kRunRegs; m < nn; m += kRunLanes) {
             const unsigned x = (unsigned)__ldcg(a.nbr + list_base(a, i) + (size_t)m * 32);
-            pair(gather4<false>(pc + (x & a.jmask)), x);
+            const float4 q = gather4<false>(pc + (x & a.jmask));
+            mixed_pair2(a, qx, qy, qz, x, q, x, q, false, acc);
         }
+        acc.settle();
         // the four lanes' exact partial sums
         auto total = [&](int x) {
 #pragma unroll
