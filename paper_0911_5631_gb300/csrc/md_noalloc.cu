@@ -92,6 +92,11 @@ __device__ __forceinline__ int gid() { return blockIdx.x * blockDim.x + threadId
 // Wrap one component into [-L/2, L/2) and return its cell coordinate (same
 // operation order as the handle-based path).
 __device__ __forceinline__ int wrap_bin(double& x, const Geo& g, int d) {
+    // |x| below L/2 by more than one part in 2^21 (high words): neither the wrap
+    // nor the folding at the faces applies, and truncation is the floor (the
+    // FP64 pipe bounds these conversions)
+    if ((__double2hiint(x) & 0x7fffffff) < __double2hiint(g.hL[d]))
+        return __double2int_rz(__dmul_rn(__dadd_rn(x, g.hL[d]), g.invW[d]));
     double s = floor(__dmul_rn(__dadd_rn(x, g.hL[d]), g.invL[d]));
     x = __dsub_rn(x, __dmul_rn(s, g.L[d]));
     int c = (int)floor(__dmul_rn(__dadd_rn(x, g.hL[d]), g.invW[d]));
@@ -216,13 +221,18 @@ __global__ void __launch_bounds__(kThreads) nz_scatter(Geo g, Scratch s) {
     if (slot >= 0 && slot < g.n) s.order[slot] = i;
 }
 
-// A thread per cell: sorts its atoms and writes them out in cell order.
+// Sorts each cell, a thread per cell, and writes the block's slots out in cell
+// order, a thread per slot (18 us for 55k cells when the cells' threads also
+// wrote their atoms out).
 __global__ void __launch_bounds__(kThreads) nz_place(Geo g, Scratch s, const double* __restrict__ pos) {
-    const int c = gid();
-    if (c >= g.ncells) return;
-    const int beg = s.start[c], end = min(s.start[c + 1], g.n);
-    if (end - beg > 1) sort_cell(s.order, beg, end);
-    for (int k = beg; k < end; k++) place_atom(g, s, pos, s.order[k], k);
+    const int c0 = blockIdx.x * kThreads, c = c0 + threadIdx.x;
+    if (c < g.ncells) {
+        const int beg = s.start[c], end = min(s.start[c + 1], g.n);
+        if (end - beg > 1) sort_cell(s.order, beg, end);
+    }
+    __syncthreads();
+    const int end = min(s.start[min(c0 + kThreads, g.ncells)], g.n);
+    for (int k = s.start[c0] + threadIdx.x; k < end; k += kThreads) place_atom(g, s, pos, s.order[k], k);
 }
 
 // All of the binning in one block, for boxes of at most kSmallAtoms atoms
@@ -309,7 +319,7 @@ __device__ __forceinline__ double reciprocal(double a) {
 // there is one, is a second run.  A thread per atom doing everything in FP64
 // as it went took 226 us for 65000 atoms and 123 us for 500 (the length of
 // one thread's chain).
-__global__ void __launch_bounds__(kThreads) nz_force(Geo g, Scratch s, double* __restrict__ f, double* __restrict__ out) {
+__global__ void __launch_bounds__(kThreads, 4) nz_force(Geo g, Scratch s, double* __restrict__ f, double* __restrict__ out) {
     __shared__ int s_queue[kAtoms * kQueue];
     __shared__ double s_sum[5][kThreads];
     __shared__ double s_uw[2][kAtoms];
@@ -384,37 +394,41 @@ __global__ void __launch_bounds__(kThreads) nz_force(Geo g, Scratch s, double* _
         const int x0 = wrapped ? (cx == 0 ? g.G[0] - 1 : 0) : max(cx - 1, 0);
         const int x1 = wrapped ? x0 : min(cx + 1, g.G[0] - 1);
         const float bx = wrapped ? (cx == 0 ? g.Lf[0] : -g.Lf[0]) : 0.0f;
-        int lo[9], hi[9];
-        float by[3], bz[3];
+        // a plane of three rows at a time, all its loads first
+        for (int dz = -1; dz <= 1; dz++) {
+            int z = cz + dz;
+            float bz = 0.0f;
+            if (z >= g.G[2]) { z -= g.G[2]; bz = -g.Lf[2]; }
+            if (z < 0) { z += g.G[2]; bz = g.Lf[2]; }
+            int lo[3], hi[3];
+            float by[3];
 #pragma unroll
-        for (int r = 0; r < 9; r++) {
-            int y = cy + r % 3 - 1, z = cz + r / 3 - 1;
-            float b = 0.0f, e = 0.0f;
-            if (y >= g.G[1]) { y -= g.G[1]; b = -g.Lf[1]; }
-            if (y < 0) { y += g.G[1]; b = g.Lf[1]; }
-            if (z >= g.G[2]) { z -= g.G[2]; e = -g.Lf[2]; }
-            if (z < 0) { z += g.G[2]; e = g.Lf[2]; }
-            by[r % 3] = b;
-            bz[r / 3] = e;
-            const int row = (z * g.G[1] + y) * g.G[0];
-            lo[r] = s.start[row + x0];
-            hi[r] = min(s.start[row + x1 + 1], g.n);
-            if (wrapped && !edge) hi[r] = lo[r];
-        }
-        float4 c[9];  // the first kLanes candidates of every row, all loads first
+            for (int r = 0; r < 3; r++) {
+                int y = cy + r - 1;
+                by[r] = 0.0f;
+                if (y >= g.G[1]) { y -= g.G[1]; by[r] = -g.Lf[1]; }
+                if (y < 0) { y += g.G[1]; by[r] = g.Lf[1]; }
+                const int row = (z * g.G[1] + y) * g.G[0];
+                lo[r] = s.start[row + x0];
+                hi[r] = min(s.start[row + x1 + 1], g.n);
+                if (wrapped && !edge) hi[r] = lo[r];
+            }
+            float4 c[3];
 #pragma unroll
-        for (int r = 0; r < 9; r++) {
-            const int t = lo[r] + sub;
-            c[r] = t < hi[r] ? s.posf[t] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        }
+            for (int r = 0; r < 3; r++) {
+                const int t = lo[r] + sub;
+                c[r] = t < hi[r] ? s.posf[t] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
 #pragma unroll
-        for (int r = 0; r < 9; r++) test(lo[r] + sub, lo[r] + sub < hi[r], c[r], r, wrapped, bx, by[r % 3], bz[r / 3]);
-#pragma unroll
-        for (int r = 0; r < 9; r++) {  // rows longer than that (few)
-            for (int t = lo[r] + sub + kLanes; __any_sync(kFull, t - sub < hi[r]); t += kLanes) {
-                const bool have = t < hi[r];
-                const float4 d = have ? s.posf[t] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                test(t, have, d, r, wrapped, bx, by[r % 3], bz[r / 3]);
+            for (int r = 0; r < 3; r++) {
+                const int row = 3 * (dz + 1) + r;
+                test(lo[r] + sub, lo[r] + sub < hi[r], c[r], row, wrapped, bx, by[r], bz);
+                // rows longer than kLanes (few)
+                for (int t = lo[r] + sub + kLanes; __any_sync(kFull, t - sub < hi[r]); t += kLanes) {
+                    const bool have = t < hi[r];
+                    const float4 d = have ? s.posf[t] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    test(t, have, d, row, wrapped, bx, by[r], bz);
+                }
             }
         }
     }
