@@ -55,7 +55,8 @@ extern "C" {
  *   positions held as FP64 cell-relative offsets, per-atom force sums in
  *   int64 fixed point (scale 2^32, independent of summation order),
  *   velocities in FP32, FP64 in the position update and the reductions.
- * MD_PREC_FP64: every arithmetic step in FP64. */
+ * MD_PREC_FP64: every arithmetic step in FP64 (an FP32 test with a margin
+ *   for its rounding only passes over pairs that lie beyond the cutoff). */
 #define MD_PREC_MIXED 0
 #define MD_PREC_FP64  1
 
@@ -80,8 +81,10 @@ typedef struct md_params {
                                  rebuild branch is a device-side conditional
                                  node (checked every third step; a step whose
                                  rebuild is due in between waits and runs
-                                 before md_step returns); 0: plain stream
-                                 launches (same results, bit for bit).         */
+                                 before md_step returns), or, for a small
+                                 system, runs its steps in one cooperative
+                                 launch; 0: plain stream launches (same
+                                 results, bit for bit).                        */
     int32_t device;           /* CUDA device ordinal; -1 (default) = current   */
     int32_t shell_bins;       /* 1 (default): the build sorts each atom's list
                                  by distance, and a step reads only the entries

@@ -8,6 +8,7 @@
 // device whether the next rebuild branch runs (cudaGraphSetConditional), so
 // no host round trip sits inside the loop, and a step whose rebuild is due
 // before the next conditional node waits (the call runs it at its end).
+// A small system's steps run in one cooperative launch instead (md_run.cuh).
 // Without graphs the same kernels are launched one by one and the host
 // reads the rebuild flag before each step.
 #include <cuda_runtime.h>
@@ -115,6 +116,7 @@ struct Sim : SimBase {
     bool profiling = false;
     std::vector<cudaEvent_t> ev;
     unsigned long long* run_words = nullptr;  // grid barrier of the one-launch step loop
+    int64_t run_closed_seen = 0;  // Counters::run_closed at the last look
     int run_blocks_max = -1;  // blocks of it that fit the device at once (-1: not yet asked)
     int64_t launches = 0;
     int64_t graph_launches = 0;
@@ -205,7 +207,7 @@ struct Sim : SimBase {
         chk(alloc(&a.part, (size_t)3 * a.nblocks));
         chk(alloc(&a.ctr, 1));
         chk(alloc(&a.d2b, (size_t)kD2Buckets * 32));
-        chk(alloc(&run_words, (size_t)4 * kRunWordStride));
+        chk(alloc(&run_words, (size_t)kRunWords));
         chk(alloc(&a.io_pos, (size_t)3 * n)); chk(alloc(&a.io_vel, (size_t)3 * n));
         if (r) return r;
         r = alloc_nbr(a.cap);
@@ -453,8 +455,6 @@ struct Sim : SimBase {
         return MD_OK;
     }
 
-    int graph_kernels_per_step() const { return 1; }
-
     // Whether plain steps run in a one-launch loop of md_run.cuh: the
     // cell-list-only variant, or the mixed form with sorted lists and the
     // default kernels, and a system whose blocks are all resident at once
@@ -498,7 +498,7 @@ struct Sim : SimBase {
         while (count > 0) {
             long long k = std::min<int64_t>(count, kRunSteps);
             void* p[] = {(void*)&a, (void*)&k, (void*)&run_words};
-            MD_CUDA(cudaMemsetAsync(run_words, 0, sizeof(unsigned long long) * 4 * kRunWordStride, stream));
+            MD_CUDA(cudaMemsetAsync(run_words, 0, sizeof(unsigned long long) * kRunWords, stream));
             MD_CUDA(cudaLaunchCooperativeKernel(run_fn(), dim3((unsigned)run_grid()), dim3(run_threads()), p, 0, stream));
             launches++;
             count -= k;
@@ -507,13 +507,14 @@ struct Sim : SimBase {
     }
 
     // Enqueues nsteps (rebuild?, force + integrate) pairs.
-    int run_steps(int64_t nsteps) {
+    // loops: plain steps may run in one-launch loops.
+    int run_steps(int64_t nsteps, bool loops = true) {
         if (nsteps <= 0) return MD_OK;
         if (prm.use_graphs && !profiling) {
             // (a plain step must not meet a call's last one: steps that wait
             // for a rebuild only leave more to run, never fewer)
             int64_t left = nsteps - 1;
-            if (left > 0 && use_run()) {
+            if (loops && left > 0 && use_run()) {
                 int r = run_loop(left);
                 if (r) return r;
                 left = 0;
@@ -632,6 +633,13 @@ struct Sim : SimBase {
 
     int finish_pending(int64_t* steps_left_out) {
         bool overflowed = false;
+        // a loop that other work on the GPU kept from starting as a whole has
+        // done nothing: the rest of this call runs as graphs
+        auto loops = [&](const Counters& c) {
+            const bool ok = c.run_closed == run_closed_seen;
+            run_closed_seen = c.run_closed;
+            return ok;
+        };
         for (int attempt = 0; attempt < 16; attempt++) {
             Counters c;
             int r = read_counters(&c);
@@ -647,14 +655,14 @@ struct Sim : SimBase {
                 r = read_counters(&c2);
                 if (r) return r;
                 if (c2.error & kErrOverflow) continue;
-                r = run_steps(c2.steps_left);
+                r = run_steps(c2.steps_left, loops(c2));
                 if (r) return r;
                 continue;
             }
             if (c.steps_left > 0 && c.error == 0) {
                 // steps that waited for a rebuild inside a graph: run them
                 // now (each round leaves fewer to wait)
-                r = run_steps(c.steps_left);
+                r = run_steps(c.steps_left, loops(c));
                 if (r) return r;
                 continue;
             }
@@ -699,6 +707,7 @@ struct Sim : SimBase {
             MD_CUDA(cudaMemcpyAsync(a.io_vel, vel, bytes, k, stream));
         }
         MD_CUDA(launch(kt.reset_counters, 1, 32, a.ctr));
+        run_closed_seen = 0;
         MD_CUDA(launch(kt.set_state, grid_atoms(), kBlock, in));
         int r = rebuild_eager();
         if (r) return r;

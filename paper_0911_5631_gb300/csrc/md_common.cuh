@@ -88,6 +88,8 @@ constexpr int kRunSteps = 2048;
 constexpr int kRunPolls = 1 << 21;
 constexpr int kRunCellBlock = 128;  // threads per block of the cell-list-only loop
 constexpr int kRunWordStride = 16;  // 64-bit words between the barrier's four words
+constexpr int kRunWords = 5 * kRunWordStride;  // ... and the gate's word after them
+constexpr int kRunGatePolls = 1 << 15;         // polls before the gate gives up (some 20 ms)
 // Elements per block of the cell-count scan (kBlock threads x 8).
 constexpr int kScanTile = 2048;
 // Largest neighbour capacity of the mixed form (its fixed-point partial
@@ -142,6 +144,7 @@ struct Counters {
     long long list_entries;    // neighbour-list length at the last build
     long long list_reads;      // entries the profiled steps read (k_count_reads)
     long long run_rebuilds;    // those of `rebuilds` done inside the one-launch step loop
+    long long run_closed;      // one-launch loops that ended at their gate, nothing done
     // reduced measurement of the last finalize
     double ke, pe, virial;
 };

@@ -92,7 +92,7 @@ inline int resolve_plan(const double box[3], int64_t n, double rc, double skin, 
     int64_t ncol = (n + 31) / 32 * 32;
     out->device_bytes = per_atom * n + 2 * pos4_b * (pair_slots(n) - n) /*pair buffers padded*/ + ncol * cap * 4 +
                         (2 * nc + 1) * 4 + ((nc + kScanTile - 1) / kScanTile) * 4 + 3 * nb * 8 +
-                        (int64_t)sizeof(Counters) + kD2Buckets * 32 * 4 + 4 * kRunWordStride * 8;
+                        (int64_t)sizeof(Counters) + kD2Buckets * 32 * 4 + kRunWords * 8;
     return MD_OK;
 }
 

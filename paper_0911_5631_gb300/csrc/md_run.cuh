@@ -70,6 +70,31 @@ struct RunBarrier {
     }
 };
 
+// The gate at the start of a loop: true in all blocks once all of them have
+// begun to run, false in all of them if that takes longer than a bounded wait
+// (the GPU is busy with other work and has room for some of the blocks only);
+// nothing has been done then, and the host takes the graphs.  *gate (zero at
+// the launch) counts the blocks that have come; the block that gives up sets
+// the top bit in the same atomic operation in which it finds the count short,
+// so every block sees either a full count without the bit or the bit.  Every
+// thread of the block must call it.
+__device__ __forceinline__ bool run_gate(unsigned* gate, int* sh, Counters* C) {
+    constexpr unsigned kShut = 0x80000000u;
+    if (threadIdx.x == 0) {
+        unsigned v = atomicAdd(gate, 1u) + 1u;
+        for (int it = 0; it < kRunGatePolls && !(v & kShut) && v != gridDim.x; it++)
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(gate) : "memory");
+        while (!(v & kShut) && v != gridDim.x) {  // (ends: another block came or this one shuts the gate)
+            const unsigned w = atomicCAS(gate, v, v | kShut);
+            if (w == v) atomicAdd((unsigned long long*)&C->run_closed, 1ull);
+            v = w == v ? kShut : w;
+        }
+        *sh = !(v & kShut);
+    }
+    __syncthreads();
+    return *sh != 0;
+}
+
 // One tile (kScanTile cells) of the exclusive scan of the cell counts, by one
 // block of any size (k_scan_apply with fewer threads).
 template <class P>
@@ -358,7 +383,7 @@ __device__ __noinline__ int run_rebuild(const Args<P>& a, int64_t i, int par, in
 
 // Up to `steps` plain steps (never a call's last one).  Cooperative launch of
 // ceil(n kRunLanes / blockDim) blocks; words: the barrier's
-// four words, zero.
+// four and the gate's, zero.
 // kB: the largest block that the instance serves (small systems have one
 // block of 128 threads on an SM and need no register limit).
 template <class P, int kB>
@@ -385,6 +410,7 @@ __global__ void __launch_bounds__(kB, kB == kRunMaxBlock ? 2 : 1) k_run(Args<P> 
     int since = since0;  // steps since the last reorder
     float d2max = 0.0f;  // the largest squared displacement that this thread has seen since the last build
     if (err0 != 0 || todo <= 0) return;
+    if (!run_gate(reinterpret_cast<unsigned*>(words + 4 * kRunWordStride), &s_sync, C)) return;
     if (threadIdx.x == 0) sa = a;
     __syncthreads();
     int rebuilds = 0, reorders = 0;
@@ -544,6 +570,7 @@ __global__ void __launch_bounds__(kRunCellBlock, 5) k_run_cells(Args<P> a, long 
     const int todo = (int)min(steps, C->steps_left - 1);  // (steps is at most kRunSteps)
     int since = (int)min(C->since_reorder, (long long)INT_MAX / 2);
     if (err0 != 0 || todo <= 0) return;
+    if (!run_gate(reinterpret_cast<unsigned*>(words + 4 * kRunWordStride), &s_sync, C)) return;
     int reorders = 0, done = 0, stop = 0;
     while (done < todo && !stop) {
         // the rebuild (k_bin .. k_rebuild_done); the grid has a thread for

@@ -1,6 +1,8 @@
 """The one-launch step loop of small systems against stream launches of the
 grid kernels, which share its arithmetic: positions and velocities are the
 same bits, and the counters the same numbers."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -89,3 +91,53 @@ def test_cells_only_loop_matches_stream_launches(n, rho, T, reorder, prec):
     for k in ("step", "rebuilds", "reorders", "max_occupancy", "ke", "pe", "virial"):
         assert a[2][k] == b[2][k], k
     assert a[2]["rebuilds"] == 1 + sum(steps)
+
+
+def test_run_loops_beside_other_work_on_the_gpu():
+    # loops of several handles and threads while an ensemble's persistent
+    # launch holds every SM: whether a loop starts as a whole or gives way to
+    # graphs, the results are those of a handle alone
+    sizes = [600, 2048, 9000, 20000]
+    states = [state(n, 0.8, 1.0, 54 + k, jitter=0.05) for k, n in enumerate(sizes)]
+    alone = [_run(p, v, L, [40, 80], 0.4) for p, v, L in states]
+    cells = [(n, state(n, 0.8, 1.0, 60, jitter=0.05)) for n in (700, 5000)]
+
+    def cells_run(n, st):
+        s = md.Simulation(st[2], n, RC, 0.0, DT, precision="fp64", cell_list_only=True)
+        s.set_state(st[0], st[1])
+        s.step(60)
+        out = s.get_state()
+        s.close()
+        return out
+
+    cells_alone = [cells_run(n, st) for n, st in cells]
+    pos, vel, L = state(16384, 0.8, 1.0, 59, jitter=0.05)
+    with md.Ensemble(2 << 30) as e:
+        e.set_shape(1024, 0, 1, 1 << 20)
+        ids = [e.add(pos, vel, L) for _ in range(160)]
+        e.run(ids, [0] * len(ids))
+        e.sync()
+        e.run(ids, [300] * len(ids))  # some tens of milliseconds on every SM
+        got, errors = {}, []
+
+        def work(key, fn):
+            try:
+                got[key] = fn()
+            except Exception as exc:  # reported below, in the test's own thread
+                errors.append(exc)
+
+        jobs = [threading.Thread(target=work, args=(k, lambda k=k: _run(*states[k], [40, 80], 0.4)))
+                for k in range(len(sizes))]
+        jobs += [threading.Thread(target=work, args=(10 + k, lambda k=k: cells_run(*cells[k])))
+                 for k in range(len(cells))]
+        for j in jobs:
+            j.start()
+        for j in jobs:
+            j.join()
+        e.sync()
+    assert not errors, errors
+    for k in range(len(sizes)):
+        assert np.array_equal(got[k][0], alone[k][0]) and np.array_equal(got[k][1], alone[k][1]), sizes[k]
+        assert got[k][2]["rebuilds"] == alone[k][2]["rebuilds"]
+    for k in range(len(cells)):
+        assert np.array_equal(got[10 + k][0], cells_alone[k][0]) and np.array_equal(got[10 + k][1], cells_alone[k][1])
