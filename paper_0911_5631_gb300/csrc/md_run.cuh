@@ -80,6 +80,7 @@ struct RunBarrier {
 // thread of the block must call it.
 __device__ __forceinline__ bool run_gate(unsigned* gate, int* sh, Counters* C) {
     constexpr unsigned kShut = 0x80000000u;
+    __syncthreads();  // the block's threads have all read the counters, which other blocks may write behind the gate
     if (threadIdx.x == 0) {
         unsigned v = atomicAdd(gate, 1u) + 1u;
         for (int it = 0; it < kRunGatePolls && !(v & kShut) && v != gridDim.x; it++)
