@@ -206,11 +206,13 @@ __device__ __forceinline__ double cell_centre(int c, double w, double hL) {
     return __dsub_rn(__dmul_rn(h, w), hL);
 }
 
-// Whether |x| is below hL by more than one part in 2^21 (the high words
-// differ): x then lies in [-L/2, L/2) and floor((x + L/2)/L) is 0, whatever
-// the rounding.  False for NaN and infinities.
+// Whether |x| is below hL by more than one part in 2^21: x then lies in
+// [-L/2, L/2), floor((x + L/2)/L) is 0 and (x + L/2) G/L stays below G,
+// whatever the rounding.  (The high words differ by two or more: where they
+// differ by one, x may be the number next to hL, whose x + L/2 rounds to L.)
+// False for NaN and infinities.
 __device__ __forceinline__ bool surely_wrapped(double x, double hL) {
-    return (__double2hiint(x) & 0x7fffffff) < __double2hiint(hL);
+    return (__double2hiint(x) & 0x7fffffff) < __double2hiint(hL) - 1;
 }
 
 template <class P>

@@ -26,6 +26,26 @@ def state(n, rho, T, seed, jitter=0.0, aspect=(1, 1, 1)):
     return pos, vel, L
 
 
+def face_state(L, spacing, seed):
+    """A simple-cubic lattice whose first planes lie on the lower faces of the
+    box L, every component on a face drawn from the numbers there and beside
+    it (both faces, one and two ulps inside, one outside), so that corners and
+    edges occur; the other components are jittered."""
+    rng = np.random.default_rng(seed)
+    L = np.broadcast_to(np.asarray(L, dtype=np.float64), (3,)).copy()
+    m = [int(x / spacing) for x in L]
+    g = np.stack(np.meshgrid(*[np.arange(k) for k in m], indexing="ij"), -1).reshape(-1, 3)
+    pos = -0.5 * L + g * (L / m) + rng.uniform(-0.04, 0.04, g.shape)
+    for k in range(3):
+        h = 0.5 * L[k]
+        inner = np.nextafter(h, 0.0)
+        beside = np.array([-h, h, inner, inner, -inner, np.nextafter(inner, 0.0), np.nextafter(h, np.inf)])
+        on = np.nonzero(g[:, k] == 0)[0]
+        pos[on, k] = beside[rng.integers(0, beside.size, on.size)]
+    pos[0] = np.nextafter(0.5 * L, 0.0)  # the corner itself
+    return pos, 0.5 * rng.standard_normal(pos.shape), L
+
+
 def sim(pos, vel, L, skin=0.4, precision="mixed", **kw):
     s = md.Simulation(L, pos.shape[0], RC, skin, DT, precision=precision, **kw)
     s.set_state(pos, vel)

@@ -7,7 +7,7 @@ import pytest
 
 import paper_0911_5631_gb300 as md
 import oracle
-from mdcheck import DT, RC, assert_trajectory_matches, ensure_built, sim, state
+from mdcheck import DT, RC, assert_trajectory_matches, ensure_built, face_state, sim, state
 
 pytestmark = pytest.mark.gpu
 
@@ -67,6 +67,19 @@ def test_replica_matches_md_step_bitwise(case):
     # both sum KE, PE and W in FP64, in different fixed orders
     for k in ("ke", "pe", "virial"):
         assert abs(m0[k] - m1[k]) <= 1e-12 * abs(m0[k]), (k, m0[k], m1[k])
+
+
+@pytest.mark.parametrize("cluster", [1, 4])
+def test_replica_with_atoms_on_the_faces_matches_md_step(cluster):
+    pos, vel, L = face_state((8.0, 16.0, 12.0), 1.12, 63)
+    p0, v0, m0 = _solo(pos, vel, L, [1, 30], 10)
+    with md.Ensemble(ARENA) as e:
+        e.set_shape(256, 0, cluster, 500)
+        rid = e.add(pos, vel, L, RC, 0.4, DT, reorder_interval=10)
+        p1, v1, m1 = _ens_run(e, rid, [1, 30])
+        assert e.status(rid) == md.MD_OK
+    assert np.array_equal(p0, p1) and np.array_equal(v0, v1)
+    assert m0["list_entries"] == m1["list_entries"] and m0["max_occupancy"] == m1["max_occupancy"]
 
 
 def test_replicas_match_oracle():

@@ -6,8 +6,8 @@ import pytest
 
 import oracle
 import paper_0911_5631_gb300 as md
-from mdcheck import (DT, FORCE_TOL, RC, assert_same_cells, assert_same_pairs, ensure_built, min_image,
-                     oracle_grid, rel_rms, sim, state, trajectory_tol)
+from mdcheck import (DT, FORCE_TOL, RC, assert_same_cells, assert_same_pairs, assert_trajectory_matches, ensure_built,
+                     face_state, min_image, oracle_grid, rel_rms, sim, state, trajectory_tol)
 
 pytestmark = pytest.mark.gpu
 
@@ -94,6 +94,33 @@ def test_loaded_positions_at_the_faces_and_far_outside(prec):
         one.get_state(ph, vh)
         assert np.array_equal(ph.numpy(), p1)
         one.close()
+
+
+# edges whose halves are short binary numbers (the number below L/2 has
+# another high word than L/2 itself) and some that are not
+FACE_BOXES = [(8.0, 10.0, 12.0), (16.0, 20.0, 12.5), (10.0, 10.3, 24.0), (9.1, 11.7, 10.9)]
+
+
+@pytest.mark.parametrize("prec", PRECS)
+@pytest.mark.parametrize("box", FACE_BOXES)
+def test_atoms_on_and_beside_the_faces(box, prec):
+    pos, vel, L = face_state(box, 1.12, 62)
+    pw = oracle.wrap(pos, L)
+    for kw in (dict(skin=0.3), dict(skin=0.0, cell_list_only=True)):
+        s = sim(pos, vel, L, precision=prec, **kw)
+        G = np.array(s.plan()["G"])
+        p, _ = s.get_state()
+        assert np.abs(min_image(p - pw, L)).max() <= 4e-16 * np.max(L)
+        assert_same_cells(s.cells(), p, L, G)
+        assert s.cells().max() < np.prod(G)
+        f_ref, _, _ = oracle.forces_cells(pw, L, oracle_grid(L, RC), RC, 1.0)
+        assert rel_rms(s.forces(), f_ref) <= FORCE_TOL[prec]
+        if kw["skin"] > 0.0:
+            assert_same_pairs(s.neighbor_pairs()[0], oracle.pairs_brute(p, L, RC + 0.3), p, L, RC + 0.3)
+        s.step(40)  # atoms cross the faces, the lists are rebuilt
+        ref = oracle.run(pw, vel, L, RC, kw["skin"], DT, 40)
+        assert_trajectory_matches(*s.get_state(), ref, L, prec, 40)
+        s.close()
 
 
 BUILDS = ["warp", "thread"]
