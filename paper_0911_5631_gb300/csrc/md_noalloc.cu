@@ -92,10 +92,11 @@ __device__ __forceinline__ int gid() { return blockIdx.x * blockDim.x + threadId
 // Wrap one component into [-L/2, L/2) and return its cell coordinate (same
 // operation order as the handle-based path).
 __device__ __forceinline__ int wrap_bin(double& x, const Geo& g, int d) {
-    // |x| below L/2 by more than one part in 2^21 (high words): neither the wrap
-    // nor the folding at the faces applies, and truncation is the floor (the
-    // FP64 pipe bounds these conversions)
-    if ((__double2hiint(x) & 0x7fffffff) < __double2hiint(g.hL[d]))
+    // |x| below L/2 by more than one part in 2^21 (high words that differ by two
+    // or more: by one, and x may be the number next to L/2, whose x + L/2 rounds
+    // to L): neither the wrap nor the folding at the faces applies, and
+    // truncation is the floor (the FP64 pipe bounds these conversions)
+    if ((__double2hiint(x) & 0x7fffffff) < __double2hiint(g.hL[d]) - 1)
         return __double2int_rz(__dmul_rn(__dadd_rn(x, g.hL[d]), g.invW[d]));
     double s = floor(__dmul_rn(__dadd_rn(x, g.hL[d]), g.invL[d]));
     x = __dsub_rn(x, __dmul_rn(s, g.L[d]));

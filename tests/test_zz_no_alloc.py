@@ -16,7 +16,7 @@ import pytest
 
 import oracle
 import paper_0911_5631_gb300 as md
-from mdcheck import FORCE_TOL, RC, ensure_built, oracle_grid, rel_rms, state
+from mdcheck import FORCE_TOL, RC, ensure_built, face_state, oracle_grid, rel_rms, state
 
 pytestmark = pytest.mark.gpu
 
@@ -121,3 +121,23 @@ def test_forces_noalloc_at_the_edges_of_its_kernels(case):
     assert np.abs(f - f_ref).max() <= 1e-12 * scale * max(1.0, n / 1000.0)
     assert u == pytest.approx(u_ref, rel=10 * FORCE_TOL["fp64"], abs=1e-12)
     assert w == pytest.approx(w_ref, rel=10 * FORCE_TOL["fp64"], abs=1e-12)
+
+
+# atoms on and beside the faces and in the corners, in boxes whose half edges
+# are short binary numbers: one block bins the first three (the third with the
+# largest number of cells that it takes), five kernels the last, whose scratch
+# then holds a larger call's atoms
+@pytest.mark.parametrize("box", [(8.0, 10.0, 12.0), (9.1, 11.7, 10.9), (18.0, 18.0, 18.0), (20.0, 24.0, 20.0)])
+def test_forces_noalloc_with_atoms_on_the_faces(box):
+    torch = pytest.importorskip("torch")
+    ensure_built()
+    big, _, Lb = state(20000, 0.8, 1.0, 22, jitter=0.1)
+    _noalloc(torch, big, Lb)
+    pos, _, L = face_state(box, 1.12, 64)
+    f_ref, u_ref, w_ref = oracle.forces_cells(oracle.wrap(pos, L), L, oracle_grid(L, RC), RC, 1.0)
+    f, u, w = _noalloc(torch, pos, L)
+    # separations within two ulps of L/2 (4e-15), a pair force's slope of up to
+    # 400 per unit (r > 1.03), six pairs an atom: 1e-11, of forces of 5 to 9
+    assert np.abs(f - f_ref).max() <= 1e-11 * np.abs(f_ref).max()
+    assert u == pytest.approx(u_ref, rel=1e-11)
+    assert w == pytest.approx(w_ref, rel=1e-11)
