@@ -394,7 +394,8 @@ struct Sim : SimBase {
     // rebuild is due waits for the next conditional node.
     int build_chunk(Chunk& c, int K, bool final_node) {
         MD_CUDA(cudaGraphCreate(&c.g, 0));
-        const int m = a.n > kRebuildEveryMaxAtoms ? 1 : kRebuildEvery;
+        // (without a skin every step is due a rebuild: each would wait)
+        const int m = a.n > kRebuildEveryMaxAtoms || skin == 0.0 ? 1 : kRebuildEvery;
         std::vector<cudaGraphConditionalHandle> h(prm.cell_list_only ? 0 : (K + m - 1) / m);
         for (auto& hh : h) MD_CUDA(cudaGraphConditionalHandleCreate(&hh, c.g, 0, 0));
         cudaGraphNode_t prev = nullptr, node = nullptr;
@@ -507,8 +508,9 @@ struct Sim : SimBase {
     }
 
     // Enqueues nsteps (rebuild?, force + integrate) pairs.
-    // loops: plain steps may run in one-launch loops.
-    int run_steps(int64_t nsteps, bool loops = true) {
+    // loops: plain steps may run in one-launch loops; single: graphs of one
+    // step only.
+    int run_steps(int64_t nsteps, bool loops = true, bool single = false) {
         if (nsteps <= 0) return MD_OK;
         if (prm.use_graphs && !profiling) {
             // (a plain step must not meet a call's last one: steps that wait
@@ -519,7 +521,7 @@ struct Sim : SimBase {
                 if (r) return r;
                 left = 0;
             }
-            for (int k = 0; k < kNumChunks; k++) {
+            for (int k = single ? kNumChunks - 1 : 0; k < kNumChunks; k++) {
                 int r = replay(plain[k], kChunks[k], false, left / kChunks[k]);
                 if (r) return r;
                 left %= kChunks[k];
@@ -640,12 +642,18 @@ struct Sim : SimBase {
             run_closed_seen = c.run_closed;
             return ok;
         };
-        for (int attempt = 0; attempt < 16; attempt++) {
+        // rounds that do not bring the call forward (an overflow regrows the
+        // lists); every other round runs at least a step
+        int idle = 0;
+        int64_t left = -1;
+        while (idle < 16) {
             Counters c;
             int r = read_counters(&c);
             if (r) return r;
             r = check_fatal(c);
             if (r) return r;
+            idle = left < 0 || c.steps_left < left ? 0 : idle + 1;
+            left = c.steps_left;
             if (c.error & kErrOverflow) {
                 overflowed = true;
                 r = regrow(c);
@@ -661,8 +669,9 @@ struct Sim : SimBase {
             }
             if (c.steps_left > 0 && c.error == 0) {
                 // steps that waited for a rebuild inside a graph: run them
-                // now (each round leaves fewer to wait)
-                r = run_steps(c.steps_left, loops(c));
+                // now (each round leaves fewer to wait; the last few take
+                // graphs of one step, which never wait)
+                r = run_steps(c.steps_left, loops(c), c.steps_left < kChunks[0]);
                 if (r) return r;
                 continue;
             }

@@ -227,3 +227,20 @@ def test_ablation_variants_give_the_same_bits(variant):
     assert np.array_equal(p0, p1) and np.array_equal(v0, v1)
     assert np.array_equal(n0[np.lexsort(n0.T[::-1])], n1[np.lexsort(n1.T[::-1])])
 
+
+# with a thin skin nearly every step asks for a rebuild, so that of a graph's
+# three steps two wait: the call has to come to its end however long it is;
+# without a skin every one does, and the graphs check before each
+@pytest.mark.parametrize("prec,skin,steps", [("fp64", 0.02, 10000), ("mixed", 0.02, 10000), ("fp64", 0.02, 47),
+                                             ("mixed", 0.02, 29), ("fp64", 0.0, 2000), ("mixed", 0.0, 34)])
+def test_a_call_whose_steps_all_rebuild_completes(prec, skin, steps):
+    pos, vel, L = state(500, 0.8, 1.0, 15, jitter=0.05)
+    out = []
+    for graphs in (True, False):
+        s = sim(pos, vel, L, skin=skin, precision=prec, shell_bins=False, use_graphs=graphs)
+        s.step(steps)
+        out.append(s.get_state() + (s.measure(),))
+        s.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    assert out[0][2]["step"] == out[1][2]["step"] == steps
+    assert out[0][2]["rebuilds"] == out[1][2]["rebuilds"] >= 0.8 * steps
