@@ -410,10 +410,11 @@ __device__ __forceinline__ double reciprocal(double a) {
     return (__double2hiint(y) & 0x7fffffff) == 0x7ff00000 ? y : r;
 }
 
-// a < b for non-negative doubles (a NaN counts as large), compared as
-// integers: a comparison on the FP64 pipe costs as much as an addition.
+// a < b for non-negative doubles, compared as integers: a comparison on the
+// FP64 pipe costs as much as an addition.  A NaN of either sign counts as
+// large (the hardware's own has its sign bit set).
 __device__ __forceinline__ bool less_bits(double a, double b) {
-    return __double_as_longlong(a) < __double_as_longlong(b);
+    return (unsigned long long)__double_as_longlong(a) < (unsigned long long)__double_as_longlong(b);
 }
 
 // Payload of a pair coordinate.  FP64 form: the position packed for the FP32
@@ -2049,7 +2050,8 @@ __device__ __forceinline__ bool kickdrift_item(const Args<P>& a, int64_t i, type
     a.ox[i] = ox; a.oy[i] = oy; a.oz[i] = oz;
     pc[i] = make_pos4(px, py, pz, pair_payload(a, P::kFp64 ? a.cell[i] : 0, px, py, pz));
     d2b = d2_bits(d2);
-    if constexpr (P::kFp64) return d2 >= a.thr2;
+    // (a NaN asks for the rebuild, which reports it)
+    if constexpr (P::kFp64) return !(d2 < a.thr2);
     else return !(d2 < a.thr2f);
 }
 
@@ -2203,8 +2205,9 @@ __device__ __forceinline__ void step_atom(const Args<P>& a, int64_t i, bool in, 
             a.ox[i] = ox; a.oy[i] = oy; a.oz[i] = oz;
             pn[i] = make_pos4(px, py, pz, pair_payload(a, P::kFp64 && !kCells ? a.cell[i] : 0, px, py, pz));
             d2b = d2_bits(d2);
-            if constexpr (P::kFp64) far = d2 >= a.thr2;
-            else far = !(d2 < a.thr2f);  // (a NaN asks for the rebuild, which reports it)
+            // (a NaN asks for the rebuild, which reports it)
+            if constexpr (P::kFp64) far = !(d2 < a.thr2);
+            else far = !(d2 < a.thr2f);
         }
     }
 }

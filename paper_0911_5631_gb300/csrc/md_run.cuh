@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(kB, kB == kRunMaxBlock ? 2 : 1) k_run(Args<P> 
                         dz = __shfl_sync(kFull, disp, lead + 2);
             const float d2 = dx * dx + dy * dy + dz * dz;
             d2max = d2 > d2max ? d2 : d2max;
-            if (d2 >= a.thr2f) say = kRunFar;
+            if (!(d2 < a.thr2f)) say = kRunFar;  // (a NaN asks for the rebuild, which reports it)
             if (acc.close) {
                 atomicOr(&C->error, kErrClose);
                 say |= kRunStop;

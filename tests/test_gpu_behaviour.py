@@ -244,3 +244,25 @@ def test_a_call_whose_steps_all_rebuild_completes(prec, skin, steps):
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
     assert out[0][2]["step"] == out[1][2]["step"] == steps
     assert out[0][2]["rebuilds"] == out[1][2]["rebuilds"] >= 0.8 * steps
+
+
+# velocities that are not finite (a rescaling whose factor overflows: infinite
+# where the atom moves, NaN where it does not) reach no result: the next step's
+# rebuild reports them, in the one-launch loops, the graphs and stream launches
+@pytest.mark.parametrize("kw", [dict(), dict(use_graphs=False), dict(shell_bins=False), dict(cell_list_only=True)])
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+def test_non_finite_velocities_are_reported(prec, kw):
+    L = np.array([9.0, 8.0, 7.0])
+    pos = np.array([[0.0, 0.0, 0.0], [3.0, 0.0, 0.0], [0.5, 2.5, -3.0]])
+    vel = np.zeros((3, 3))
+    vel[1, 0] = 1e-20
+    for steps in (1, 2, 40):
+        s = sim(pos, vel, L, skin=0.0 if "cell_list_only" in kw else 0.4, precision=prec, **kw)
+        s.rescale(1e300)
+        with pytest.raises(md.MDError) as e:
+            s.step(steps)
+        assert e.value.code == md.MD_EUNSTABLE and "non-finite" in str(e.value)
+        s.set_state(pos, vel)
+        s.step(steps)
+        assert np.all(np.isfinite(s.get_state()[0]))
+        s.close()
