@@ -11,6 +11,7 @@
 // A small system's steps run in one cooperative launch instead (md_run.cuh).
 // Without graphs the same kernels are launched one by one and the host
 // reads the rebuild flag before each step.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -41,6 +42,26 @@ thread_local std::string g_create_error;
 // the energy kernel.
 constexpr int kChunks[] = {10 * kRebuildEvery, kRebuildEvery, 1};
 constexpr int kNumChunks = sizeof(kChunks) / sizeof(kChunks[0]);
+
+// Whether the `bytes` bytes at device address p lie within one allocation
+// (what a copy checks of its arguments, and a kernel does not).
+bool within_allocation(const void* p, size_t bytes) {
+    using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Range range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (Range)f;
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = (CUdeviceptr)(uintptr_t)p;
+    return range && range(&base, &size, at) == CUDA_SUCCESS && at - base <= size && bytes <= size - (at - base);
+}
 
 // Zeroed storage for cudaGraphNodeParams (its union has no default
 // constructor).
@@ -688,15 +709,17 @@ struct Sim : SimBase {
 
     // ---- API -------------------------------------------------------------
 
-    // Whether a kernel may use the caller's array in place of a staged copy:
-    // memory of this device, aligned to its elements.
+    // Whether a kernel may use the caller's array of n x 3 doubles in place of a
+    // staged copy: memory of this device, aligned to its elements, all of it in
+    // one allocation (a copy refuses an array that is too short).
     bool direct(const void* p) const {
         cudaPointerAttributes at;
         if (((uintptr_t)p & 7u) != 0 || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
-        return at.type == cudaMemoryTypeDevice && at.device == this->device;
+        return at.type == cudaMemoryTypeDevice && at.device == this->device &&
+               within_allocation(p, sizeof(double) * 3 * (size_t)a.n);
     }
 
     int set_state(const double* pos, const double* vel, bool device) override {

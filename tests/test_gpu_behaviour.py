@@ -1,5 +1,7 @@
 """Determinism, reordering, capacity growth, error reporting and energy
 conservation of the CUDA path (through the C ABI)."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -266,3 +268,30 @@ def test_non_finite_velocities_are_reported(prec, kw):
         s.step(steps)
         assert np.all(np.isfinite(s.get_state()[0]))
         s.close()
+
+
+def test_a_device_array_that_is_too_short_is_refused():
+    torch = pytest.importorskip("torch")
+    n = 100
+    pos, vel, L = state(n, 0.5, 1.0, 16, jitter=0.05)
+    s = sim(pos, vel, L)
+    torch.zeros(1, device="cuda")  # the device's context is current in this thread
+    cu = ctypes.CDLL("libcuda.so.1")
+    short = ctypes.c_uint64()
+    assert cu.cuMemAlloc_v2(ctypes.byref(short), ctypes.c_size_t(1024)) == 0
+    try:
+        # the driver hands memory out in pages of 2 MB: the rest of the array is
+        # mapped, whoever holds it
+        if short.value % (1 << 21) + 24 * n > 1 << 21:
+            pytest.skip("the allocation lies at the end of its page")
+        full = torch.tensor(vel, device="cuda")
+        torch.cuda.synchronize()
+        for p, v in ((short.value, full.data_ptr()), (full.data_ptr(), short.value)):
+            with pytest.raises(md.MDError) as e:
+                md.md_set_state_device(s.h, p, v)
+            assert e.value.code == md.MD_ECUDA
+    finally:
+        assert cu.cuMemFree_v2(short) == 0
+    s.set_state(pos, vel)
+    s.step(10)
+    s.close()
