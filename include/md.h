@@ -248,6 +248,17 @@ int md_debug_cells(md_handle* h, int32_t* cell);
 int md_debug_neighbors(md_handle* h, int64_t* count, int64_t* entries, int32_t* pairs,
                        int64_t capacity);
 
+/* Test aid for the one-launch step loops of small systems.  hold: 0 as ever,
+ * MD_HOLD_GATE: loops do not start as a whole (as when other work fills the
+ * GPU) and md_step takes its graphs, MD_HOLD_BARRIER: their first grid
+ * barrier runs out of time (about a second) and md_step returns MD_ECUDA; the
+ * handle works again after md_set_state.  counts (may be NULL): loops
+ * launched since md_create, steps that they ran and loops that did not start
+ * since md_set_state. */
+#define MD_HOLD_GATE    1
+#define MD_HOLD_BARRIER 2
+int md_debug_loop(md_handle* h, int32_t hold, int64_t counts[3]);
+
 /* Plan of an existing handle (current capacity included). */
 int md_get_plan(md_handle* h, md_plan_t* out);
 

@@ -156,6 +156,7 @@ SIGNATURES = [
     ("md_debug_cells", C.c_int, [_H, C.c_void_p]),
     ("md_debug_neighbors", C.c_int, [_H, C.POINTER(C.c_int64), C.POINTER(C.c_int64), C.c_void_p,
                                      C.c_int64]),
+    ("md_debug_loop", C.c_int, [_H, C.c_int32, C.POINTER(C.c_int64)]),
     ("md_get_plan", C.c_int, [_H, C.POINTER(md_plan_t)]),
     ("md_set_profiling", C.c_int, [_H, C.c_int]),
     ("md_kernel_stats", C.c_int, [_H, C.POINTER(md_kernel_stats_t)]),
@@ -186,6 +187,7 @@ SIGNATURES = [
     ("md_strerror", C.c_char_p, [C.c_int]),
 ]
 
+MD_HOLD_GATE, MD_HOLD_BARRIER = 1, 2
 MD_NOALLOC_MAX_ATOMS = 65536
 MD_NOALLOC_MAX_CELLS = 65536
 
@@ -310,6 +312,14 @@ def md_debug_neighbors(h):
     pairs = np.empty((max(cnt.value, 1), 2), dtype=np.int32)
     _check(lib().md_debug_neighbors(h, C.byref(cnt), C.byref(ent), pairs.ctypes.data, cnt.value), h)
     return pairs[:cnt.value], ent.value
+
+
+def md_debug_loop(h, hold=0):
+    """Sets `hold` (MD_HOLD_*, 0: none); returns (loops launched, steps that
+    they ran, loops that did not start)."""
+    c = (C.c_int64 * 3)()
+    _check(lib().md_debug_loop(h, int(hold), c), h)
+    return tuple(c)
 
 
 def md_get_plan(h) -> md_plan_t:

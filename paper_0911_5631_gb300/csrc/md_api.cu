@@ -93,6 +93,7 @@ struct SimBase {
     virtual int get_forces(double* f) = 0;
     virtual int debug_cells(int32_t* cell) = 0;
     virtual int debug_neighbors(int64_t* count, int64_t* entries, int32_t* pairs, int64_t cap) = 0;
+    virtual int debug_loop(int hold, int64_t counts[3]) = 0;
     virtual int get_plan(md_plan_t* out) = 0;
     virtual int set_profiling(int on) = 0;
     virtual int kernel_stats(md_kernel_stats_t* out) = 0;
@@ -138,9 +139,11 @@ struct Sim : SimBase {
     std::vector<cudaEvent_t> ev;
     unsigned long long* run_words = nullptr;  // grid barrier of the one-launch step loop
     int64_t run_closed_seen = 0;  // Counters::run_closed at the last look
+    int hold = 0;                 // MD_HOLD_*, set by a test
     int run_blocks_max = -1;  // blocks of it that fit the device at once (-1: not yet asked)
     int64_t launches = 0;
     int64_t graph_launches = 0;
+    int64_t loops_launched = 0;
     int64_t steps_run = 0;
     int64_t rebuilds_at_mark = 0;
     double step_ms = 0.0;
@@ -521,8 +524,13 @@ struct Sim : SimBase {
             long long k = std::min<int64_t>(count, kRunSteps);
             void* p[] = {(void*)&a, (void*)&k, (void*)&run_words};
             MD_CUDA(cudaMemsetAsync(run_words, 0, sizeof(unsigned long long) * kRunWords, stream));
+            // (held for a test: a count that never comes to the number of blocks)
+            for (int w = 0; w < 4 && hold == MD_HOLD_BARRIER; w++)
+                MD_CUDA(cudaMemsetAsync(run_words + w * kRunWordStride, 0x20, 2, stream));
+            if (hold == MD_HOLD_GATE) MD_CUDA(cudaMemsetAsync(run_words + 4 * kRunWordStride, 0x20, 2, stream));
             MD_CUDA(cudaLaunchCooperativeKernel(run_fn(), dim3((unsigned)run_grid()), dim3(run_threads()), p, 0, stream));
             launches++;
+            loops_launched++;
             count -= k;
         }
         return MD_OK;
@@ -621,6 +629,14 @@ struct Sim : SimBase {
     }
 
     int check_fatal(const Counters& c) {
+        if (c.error & kErrWait) {
+            // (the loop may have left a binning half done: the counts are zero
+            // again for the next one)
+            MD_CUDA(cudaMemsetAsync(a.count, 0, sizeof(int) * a.ncells, stream));
+            MD_CUDA(cudaMemsetAsync(a.tile_sum, 0, sizeof(int) * a.ntiles, stream));
+            err = "a grid barrier of the one-launch step loop ran out of time";
+            return MD_ECUDA;
+        }
         if (c.error & kErrInternal) {
             err = "internal: a step kernel without the final-step path met the last step of a call";
             return MD_ECUDA;
@@ -956,6 +972,23 @@ struct Sim : SimBase {
         return MD_OK;
     }
 
+    int debug_loop(int hold_, int64_t counts[3]) override {
+        DevGuard dg(device);
+        if (hold_ < 0 || hold_ > MD_HOLD_BARRIER) {
+            err = "unknown hold";
+            return MD_EINVAL;
+        }
+        hold = hold_;
+        if (!counts) return MD_OK;
+        Counters c;
+        int r = read_counters(&c);
+        if (r) return r;
+        counts[0] = loops_launched;
+        counts[1] = c.run_steps;
+        counts[2] = c.run_closed;
+        return MD_OK;
+    }
+
     int set_profiling(int on) override {
         profiling = on != 0;
         return MD_OK;
@@ -1102,6 +1135,10 @@ int md_debug_cells(md_handle* h, int32_t* cell) {
 int md_debug_neighbors(md_handle* h, int64_t* count, int64_t* entries, int32_t* pairs, int64_t capacity) {
     MD_HANDLE_CHECK(h);
     return h->sim->debug_neighbors(count, entries, pairs, capacity);
+}
+int md_debug_loop(md_handle* h, int32_t hold, int64_t counts[3]) {
+    MD_HANDLE_CHECK(h);
+    return h->sim->debug_loop(hold, counts);
 }
 int md_get_plan(md_handle* h, md_plan_t* out) {
     MD_HANDLE_CHECK(h);

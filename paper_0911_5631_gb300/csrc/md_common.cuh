@@ -113,6 +113,7 @@ enum : int {
     kErrUnstable = 2,   // non-finite coordinate or velocity
     kErrClose = 4,      // pair closer than the fixed-point range allows
     kErrInternal = 8,   // a plain step node met the last step of a call
+    kErrWait = 16,      // a grid barrier of a one-launch loop ran out of time
 };
 
 // Step-kernel modes.
@@ -144,6 +145,7 @@ struct Counters {
     long long list_entries;    // neighbour-list length at the last build
     long long list_reads;      // entries the profiled steps read (k_count_reads)
     long long run_rebuilds;    // those of `rebuilds` done inside the one-launch step loop
+    long long run_steps;       // steps done inside it
     long long run_closed;      // one-launch loops that ended at their gate, nothing done
     // reduced measurement of the last finalize
     double ke, pe, virial;

@@ -38,7 +38,8 @@ constexpr int kRunStop = 2;  // an error: end the run
 // it is used again three barriers later.  (A word per block, polled by all
 // blocks, took 3.7 us at 64 blocks and 6.5 us at 209: the polls queue at the
 // few lines that hold the words.)  The wait is bounded (about a second): a
-// block that gives up records kErrInternal and stops.
+// block that gives up records kErrWait and sees kRunStop, at which it leaves
+// the loop without another barrier.
 struct RunBarrier {
     unsigned long long* words;
     unsigned epoch;
@@ -58,7 +59,7 @@ struct RunBarrier {
             } while (((unsigned)x & 0xffffu) != gridDim.x && ++it < kRunPolls);
             int got = ((unsigned)x >> 16 ? kRunFar : 0) | ((unsigned)(x >> 32) ? kRunStop : 0);
             if (((unsigned)x & 0xffffu) != gridDim.x) {
-                atomicOr(&C->error, kErrInternal);
+                atomicOr(&C->error, kErrWait);
                 got = kRunStop;
             }
             asm volatile("fence.acq_rel.gpu;" ::: "memory");
@@ -329,7 +330,7 @@ __device__ __forceinline__ int run_build(const Args<P>& a, int64_t s, bool in, i
 // The rebuild branch (k_bin .. k_rebuild_done) of the loop: seven barriers with
 // a reorder, four without.  A cell's atoms keep their order of arrival unless
 // the atoms are reordered: nothing in the mixed form depends on it.  Returns
-// what its barriers said.  (A function of its own, so that its
+// what its last barrier said.  (A function of its own, so that its
 // registers do not weigh on the loop's.)
 template <class P, int kB>
 __device__ __noinline__ int run_rebuild(const Args<P>& a, int64_t i, int par, int reorder, RunBarrier bar, int2* stage,
@@ -352,21 +353,29 @@ __device__ __noinline__ int run_rebuild(const Args<P>& a, int64_t i, int par, in
     }
     const unsigned peers = __match_any_sync(kFull, tile);
     if (tile >= 0 && lane == __ffs(peers) - 1) atomicAdd(&a.tile_sum[tile], __popc(peers));
+    // (no block says anything before the last barrier: a stop is a wait that
+    // ran out)
     int said = bar.sync(0, s_sync, C);
+    if (said & kRunStop) return said;
     for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) run_scan_tile(a, t, s_scan);
-    said |= bar.sync(0, s_sync, C);
+    said = bar.sync(0, s_sync, C);
+    if (said & kRunStop) return said;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, dt = (int64_t)gridDim.x * blockDim.x;
     if (in && sub == 0) scatter_item<P>(a, i, reorder);
     for (int64_t c = t0; c < a.ncells; c += dt) a.count[c] = 0;
     for (int64_t c = t0; c < a.ntiles; c += dt) a.tile_sum[c] = 0;
-    said |= bar.sync(0, s_sync, C);
+    said = bar.sync(0, s_sync, C);
+    if (said & kRunStop) return said;
     if (reorder) {
         for (int64_t c = t0; c < a.ncells; c += dt) cellsort_item<P>(a, c);
-        said |= bar.sync(0, s_sync, C);
+        said = bar.sync(0, s_sync, C);
+        if (said & kRunStop) return said;
         if (in && sub == 0) gather_item<P>(a, i, reorder);
-        said |= bar.sync(0, s_sync, C);
+        said = bar.sync(0, s_sync, C);
+        if (said & kRunStop) return said;
         if (in && sub == 0) commit_item<P>(a, i, par);
-        said |= bar.sync(0, s_sync, C);
+        said = bar.sync(0, s_sync, C);
+        if (said & kRunStop) return said;
     }
     const int m = run_build<P, kB == kRunMaxBlock ? 1 : 3>(a, i, in, stage, (int)blockDim.x);
     const int wmax = __reduce_max_sync(kFull, m);
@@ -376,10 +385,8 @@ __device__ __noinline__ int run_rebuild(const Args<P>& a, int64_t i, int par, in
         atomicAdd((unsigned long long*)&C->list_entries, (unsigned long long)wsum);
     }
     // an error of the binning (recorded before an earlier barrier) or
-    // of this thread's list stops the run, for all blocks alike; so
-    // does a barrier that gave up
-    said |= bar.sync(m > a.cap || __ldcg(&C->error) != 0 ? kRunStop : 0, s_sync, C);
-    return said;
+    // of this thread's list stops the run, for all blocks alike
+    return bar.sync(m > a.cap || __ldcg(&C->error) != 0 ? kRunStop : 0, s_sync, C);
 }
 
 // Up to `steps` plain steps (never a call's last one).  Cooperative launch of
@@ -540,6 +547,7 @@ __global__ void __launch_bounds__(kB, kB == kRunMaxBlock ? 2 : 1) k_run(Args<P> 
         C->reorder_now = reorder;
         C->steps_left -= done;
         C->step += done;
+        C->run_steps += done;
         C->since_reorder = reorders > 0 ? since : C->since_reorder + done;
         C->rebuilds += rebuilds;
         C->run_rebuilds += rebuilds;
@@ -585,23 +593,25 @@ __global__ void __launch_bounds__(kRunCellBlock, 5) k_run_cells(Args<P> a, long 
         }
         const unsigned peers = __match_any_sync(0xffffffffu, tile);
         if (tile >= 0 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&a.tile_sum[tile], __popc(peers));
-        bar.sync(0, &s_sync, C);
+        // (no block says anything before a step's last barrier: a stop is a
+        // wait that ran out)
+        if (bar.sync(0, &s_sync, C) & kRunStop) break;
         for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) run_scan_tile(a, t, s_scan);
-        bar.sync(0, &s_sync, C);
+        if (bar.sync(0, &s_sync, C) & kRunStop) break;
         if (t0 < a.n) scatter_item<P>(a, t0, reorder);
         for (int64_t c = t0; c < a.ncells; c += dt) a.count[c] = 0;
         for (int64_t c = t0; c < a.ntiles; c += dt) a.tile_sum[c] = 0;
-        bar.sync(0, &s_sync, C);
+        if (bar.sync(0, &s_sync, C) & kRunStop) break;
         if (sorts_cells<P>(reorder)) {
             for (int64_t c = t0; c < a.ncells; c += dt) {
                 cellsort_item<P>(a, c);
                 const int end = min(a.cell_start[c + 1], (int)a.n);
                 for (int s = a.cell_start[c]; s < end; s++) gather_item<P>(a, s, reorder);
             }
-            bar.sync(0, &s_sync, C);
+            if (bar.sync(0, &s_sync, C) & kRunStop) break;
             if (reorder) {
                 if (t0 < a.n) commit_item<P>(a, t0, par);
-                bar.sync(0, &s_sync, C);
+                if (bar.sync(0, &s_sync, C) & kRunStop) break;
                 reorders++;
                 since = 0;
             }
@@ -638,6 +648,7 @@ __global__ void __launch_bounds__(kRunCellBlock, 5) k_run_cells(Args<P> a, long 
         C->reorder_now = reorder;
         C->steps_left -= done;
         C->step += done;
+        C->run_steps += done;
         C->since_reorder = reorders > 0 ? since : C->since_reorder + done;
         C->rebuilds += done;
         C->run_rebuilds += done;

@@ -2,6 +2,7 @@
 grid kernels, which share its arithmetic: positions and velocities are the
 same bits, and the counters the same numbers."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -141,3 +142,45 @@ def test_run_loops_beside_other_work_on_the_gpu():
         assert got[k][2]["rebuilds"] == alone[k][2]["rebuilds"]
     for k in range(len(cells)):
         assert np.array_equal(got[10 + k][0], cells_alone[k][0]) and np.array_equal(got[10 + k][1], cells_alone[k][1])
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(cell_list_only=True), dict(cell_list_only=True, precision="fp64")])
+def test_a_barrier_that_runs_out_ends_the_loop(kw):
+    # the first barrier of a loop never fills: of a rebuild (the state is hot:
+    # its atoms have moved skin/2 when the loop starts; cells only, every step)
+    n = 500
+    pos, vel, L = state(n, 0.8, 1.0, 55, jitter=0.05)
+    skin = 0.0 if kw else 0.01
+    s = md.Simulation(L, n, RC, skin, DT, **kw)
+    s.set_state(pos, vel)
+    md.md_debug_loop(s.h, md.MD_HOLD_BARRIER)
+    t = time.perf_counter()
+    with pytest.raises(md.MDError) as e:
+        s.step(20)
+    t = time.perf_counter() - t
+    assert e.value.code == md.MD_ECUDA and "barrier" in str(e.value)
+    assert t < 1.7 * _one_wait(L, n, pos, vel), t  # one wait, not one at each barrier of the rebuild
+    assert md.md_debug_loop(s.h)[1] == 0
+    s.set_state(pos, vel)
+    s.step(20)
+    p, v = s.get_state()
+    assert md.md_debug_loop(s.h)[1] == 19
+    s.close()
+    b = md.Simulation(L, n, RC, skin, DT, use_graphs=False, **kw)
+    b.set_state(pos, vel)
+    b.step(20)
+    assert all(np.array_equal(x, y) for x, y in zip((p, v), b.get_state()))
+    b.close()
+
+
+def _one_wait(L, n, pos, vel):
+    # a step's own barrier, the only one that a loop with a good list meets
+    s = md.Simulation(L, n, RC, 0.4, DT)
+    s.set_state(pos, vel)
+    md.md_debug_loop(s.h, md.MD_HOLD_BARRIER)
+    t = time.perf_counter()
+    with pytest.raises(md.MDError):
+        s.step(3)
+    t = time.perf_counter() - t
+    s.close()
+    return t
