@@ -251,7 +251,7 @@ int md_debug_neighbors(md_handle* h, int64_t* count, int64_t* entries, int32_t* 
 /* Test aid for the one-launch step loops of small systems.  hold: 0 as ever,
  * MD_HOLD_GATE: loops do not start as a whole (as when other work fills the
  * GPU) and md_step takes its graphs, MD_HOLD_BARRIER: their first grid
- * barrier runs out of time (about a second) and md_step returns MD_ECUDA; the
+ * barrier runs out of time (0.33 s) and md_step returns MD_ECUDA; the
  * handle works again after md_set_state.  counts (may be NULL): loops
  * launched since md_create, steps that they ran and loops that did not start
  * since md_set_state. */

@@ -140,6 +140,9 @@ struct Sim : SimBase {
     unsigned long long* run_words = nullptr;  // grid barrier of the one-launch step loop
     int64_t run_closed_seen = 0;  // Counters::run_closed at the last look
     int hold = 0;                 // MD_HOLD_*, set by a test
+    bool run_shut = false;        // a loop of the running call did not start
+    int run_rest = 0;             // calls that take graphs before the next loop
+    int run_backoff = 0;          // ... after the last one that did not start
     int run_blocks_max = -1;  // blocks of it that fit the device at once (-1: not yet asked)
     int64_t launches = 0;
     int64_t graph_launches = 0;
@@ -522,7 +525,8 @@ struct Sim : SimBase {
     int run_loop(int64_t count) {
         while (count > 0) {
             long long k = std::min<int64_t>(count, kRunSteps);
-            void* p[] = {(void*)&a, (void*)&k, (void*)&run_words};
+            long long closed = run_closed_seen;
+            void* p[] = {(void*)&a, (void*)&k, (void*)&run_words, (void*)&closed};
             MD_CUDA(cudaMemsetAsync(run_words, 0, sizeof(unsigned long long) * kRunWords, stream));
             // (held for a test: a count that never comes to the number of blocks)
             for (int w = 0; w < 4 && hold == MD_HOLD_BARRIER; w++)
@@ -539,7 +543,7 @@ struct Sim : SimBase {
     // Enqueues nsteps (rebuild?, force + integrate) pairs.
     // loops: plain steps may run in one-launch loops; single: graphs of one
     // step only.
-    int run_steps(int64_t nsteps, bool loops = true, bool single = false) {
+    int run_steps(int64_t nsteps, bool loops, bool single = false) {
         if (nsteps <= 0) return MD_OK;
         if (prm.use_graphs && !profiling) {
             // (a plain step must not meet a call's last one: steps that wait
@@ -670,14 +674,20 @@ struct Sim : SimBase {
         return rebuild_eager();
     }
 
-    int finish_pending(int64_t* steps_left_out) {
+    // loops: as in run_steps
+    int finish_pending(int64_t* steps_left_out, bool loops) {
         bool overflowed = false;
         // a loop that other work on the GPU kept from starting as a whole has
         // done nothing: the rest of this call runs as graphs
-        auto loops = [&](const Counters& c) {
-            const bool ok = c.run_closed == run_closed_seen;
-            run_closed_seen = c.run_closed;
-            return ok;
+        auto look = [&](Counters* c) {
+            int r = read_counters(c);
+            if (r) return r;
+            if (c->run_closed != run_closed_seen) {
+                run_closed_seen = c->run_closed;
+                run_shut = true;
+                loops = false;
+            }
+            return (int)MD_OK;
         };
         // rounds that do not bring the call forward (an overflow regrows the
         // lists); every other round runs at least a step
@@ -685,7 +695,7 @@ struct Sim : SimBase {
         int64_t left = -1;
         while (idle < 16) {
             Counters c;
-            int r = read_counters(&c);
+            int r = look(&c);
             if (r) return r;
             r = check_fatal(c);
             if (r) return r;
@@ -697,10 +707,10 @@ struct Sim : SimBase {
                 if (r) return r;
                 // the step that met the overflow has not run yet
                 Counters c2;
-                r = read_counters(&c2);
+                r = look(&c2);
                 if (r) return r;
                 if (c2.error & kErrOverflow) continue;
-                r = run_steps(c2.steps_left, loops(c2));
+                r = run_steps(c2.steps_left, loops);
                 if (r) return r;
                 continue;
             }
@@ -708,7 +718,7 @@ struct Sim : SimBase {
                 // steps that waited for a rebuild inside a graph: run them
                 // now (each round leaves fewer to wait; the last few take
                 // graphs of one step, which never wait)
-                r = run_steps(c.steps_left, loops(c), c.steps_left < kChunks[0]);
+                r = run_steps(c.steps_left, loops, c.steps_left < kChunks[0]);
                 if (r) return r;
                 continue;
             }
@@ -789,11 +799,19 @@ struct Sim : SimBase {
         }
         long long nn = (long long)n;
         MD_CUDA(launch(kt.kickdrift, grid_atoms(), kBlock, a, nn));
-        int r = run_steps(n);
+        // After a loop that could not start, calls take graphs at once for a
+        // while: a wait at the gate for each would cost more than the loops give.
+        const bool loops = run_rest == 0;
+        const int64_t launched = loops_launched;
+        if (run_rest > 0) run_rest--;
+        run_shut = false;
+        int r = run_steps(n, loops);
         if (r) return r;
         int64_t left = 0;
-        r = finish_pending(&left);
+        r = finish_pending(&left, loops);
         if (r) return r;
+        if (run_shut) run_rest = run_backoff = run_backoff ? std::min(2 * run_backoff, kRunRestMax) : 1;
+        else if (loops_launched != launched) run_backoff = 0;
         if (left != 0) {
             err = "step counter did not reach zero";
             return MD_ECUDA;

@@ -83,13 +83,16 @@ constexpr int kRunLanes = 4;
 constexpr int kRunMaxBlock = 384;
 constexpr int kRunMaxBlocks = 304;
 // Steps of one such launch at most (some milliseconds), and polls of a word
-// before a wait is given up (at half a microsecond or more each).
+// before a wait is given up (0.16 us each).
 constexpr int kRunSteps = 2048;
 constexpr int kRunPolls = 1 << 21;
 constexpr int kRunCellBlock = 128;  // threads per block of the cell-list-only loop
 constexpr int kRunWordStride = 16;  // 64-bit words between the barrier's four words
 constexpr int kRunWords = 5 * kRunWordStride;  // ... and the gate's word after them
-constexpr int kRunGatePolls = 1 << 15;         // polls before the gate gives up (some 20 ms)
+constexpr int kRunGatePolls = 1 << 12;         // polls before the gate gives up (0.65 ms)
+// Calls of md_step that take graphs at once after one whose loop did not start:
+// 1, then twice as many each time up to this, until a loop starts again.
+constexpr int kRunRestMax = 64;
 // Elements per block of the cell-count scan (kBlock threads x 8).
 constexpr int kScanTile = 2048;
 // Largest neighbour capacity of the mixed form (its fixed-point partial

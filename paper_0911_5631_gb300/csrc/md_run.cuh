@@ -37,7 +37,7 @@ constexpr int kRunStop = 2;  // an error: end the run
 // word of the barrier before the one just passed, which every block has left;
 // it is used again three barriers later.  (A word per block, polled by all
 // blocks, took 3.7 us at 64 blocks and 6.5 us at 209: the polls queue at the
-// few lines that hold the words.)  The wait is bounded (about a second): a
+// few lines that hold the words.)  The wait is bounded (0.33 s): a
 // block that gives up records kErrWait and sees kRunStop, at which it leaves
 // the loop without another barrier.
 struct RunBarrier {
@@ -78,12 +78,17 @@ struct RunBarrier {
 // the launch) counts the blocks that have come; the block that gives up sets
 // the top bit in the same atomic operation in which it finds the count short,
 // so every block sees either a full count without the bit or the bit.  Every
-// thread of the block must call it.
-__device__ __forceinline__ bool run_gate(unsigned* gate, int* sh, Counters* C) {
+// thread of the block must call it.  closed: Counters::run_closed when the host
+// queued the loop; a loop behind one that has not started, of the same call,
+// does not start either, at once.  (A block that reads the count after another
+// of its own launch has shut the gate finds it shut either way.)
+__device__ __forceinline__ bool run_gate(unsigned* gate, int* sh, Counters* C, long long closed) {
     constexpr unsigned kShut = 0x80000000u;
     __syncthreads();  // the block's threads have all read the counters, which other blocks may write behind the gate
     if (threadIdx.x == 0) {
-        unsigned v = atomicAdd(gate, 1u) + 1u;
+        long long now;
+        asm volatile("ld.relaxed.gpu.global.s64 %0, [%1];" : "=l"(now) : "l"(&C->run_closed) : "memory");
+        unsigned v = now != closed ? kShut : atomicAdd(gate, 1u) + 1u;
         for (int it = 0; it < kRunGatePolls && !(v & kShut) && v != gridDim.x; it++)
             asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(gate) : "memory");
         while (!(v & kShut) && v != gridDim.x) {  // (ends: another block came or this one shuts the gate)
@@ -395,7 +400,8 @@ __device__ __noinline__ int run_rebuild(const Args<P>& a, int64_t i, int par, in
 // kB: the largest block that the instance serves (small systems have one
 // block of 128 threads on an SM and need no register limit).
 template <class P, int kB>
-__global__ void __launch_bounds__(kB, kB == kRunMaxBlock ? 2 : 1) k_run(Args<P> a, long long steps, unsigned long long* words) {
+__global__ void __launch_bounds__(kB, kB == kRunMaxBlock ? 2 : 1) k_run(Args<P> a, long long steps, unsigned long long* words,
+                                                                                  long long closed) {
     static_assert(!P::kFp64, "mixed form only");
     __shared__ int2 s_stage[kRunStage * kB];
     __shared__ int s_sync;
@@ -418,7 +424,7 @@ __global__ void __launch_bounds__(kB, kB == kRunMaxBlock ? 2 : 1) k_run(Args<P> 
     int since = since0;  // steps since the last reorder
     float d2max = 0.0f;  // the largest squared displacement that this thread has seen since the last build
     if (err0 != 0 || todo <= 0) return;
-    if (!run_gate(reinterpret_cast<unsigned*>(words + 4 * kRunWordStride), &s_sync, C)) return;
+    if (!run_gate(reinterpret_cast<unsigned*>(words + 4 * kRunWordStride), &s_sync, C, closed)) return;
     if (threadIdx.x == 0) sa = a;
     __syncthreads();
     int rebuilds = 0, reorders = 0;
@@ -563,7 +569,8 @@ __global__ void __launch_bounds__(kB, kB == kRunMaxBlock ? 2 : 1) k_run(Args<P> 
 // order, so the results are the same bits.  Cooperative launch of
 // ceil(n kCellLanes / kRunCellBlock) blocks.
 template <class P>
-__global__ void __launch_bounds__(kRunCellBlock, 5) k_run_cells(Args<P> a, long long steps, unsigned long long* words) {
+__global__ void __launch_bounds__(kRunCellBlock, 5) k_run_cells(Args<P> a, long long steps, unsigned long long* words,
+                                                             long long closed) {
     using real = typename P::real;
     __shared__ int s_queue[P::kFp64 ? kRunCellBlock / kCellLanes * kCellQueue : 1];
     __shared__ int s_sync;
@@ -579,7 +586,7 @@ __global__ void __launch_bounds__(kRunCellBlock, 5) k_run_cells(Args<P> a, long 
     const int todo = (int)min(steps, C->steps_left - 1);  // (steps is at most kRunSteps)
     int since = (int)min(C->since_reorder, (long long)INT_MAX / 2);
     if (err0 != 0 || todo <= 0) return;
-    if (!run_gate(reinterpret_cast<unsigned*>(words + 4 * kRunWordStride), &s_sync, C)) return;
+    if (!run_gate(reinterpret_cast<unsigned*>(words + 4 * kRunWordStride), &s_sync, C, closed)) return;
     int reorders = 0, done = 0, stop = 0;
     while (done < todo && !stop) {
         // the rebuild (k_bin .. k_rebuild_done); the grid has a thread for

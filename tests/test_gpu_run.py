@@ -184,3 +184,28 @@ def _one_wait(L, n, pos, vel):
     t = time.perf_counter() - t
     s.close()
     return t
+
+
+def test_a_loop_that_cannot_start_gives_way_to_graphs():
+    n = 3000
+    pos, vel, L = state(n, 0.8, 1.5, 56, jitter=0.05)
+    ref = _run(pos, vel, L, [40] * 8 + [5000] + [40] * 8, 0.4, use_graphs=False)
+    s = md.Simulation(L, n, RC, 0.4, DT)
+    s.set_state(pos, vel)
+    md.md_debug_loop(s.h, md.MD_HOLD_GATE)
+    for _ in range(8):
+        s.step(40)
+    # the first, third and sixth call tried; no step ran in a loop
+    assert md.md_debug_loop(s.h, md.MD_HOLD_GATE) == (3, 0, 3)
+    s.step(5000)  # (a call that takes graphs at once: the fourth after the sixth is the next to try)
+    assert md.md_debug_loop(s.h, 0) == (3, 0, 3)
+    for _ in range(8):
+        s.step(40)
+    launched, steps, shut = md.md_debug_loop(s.h)
+    assert shut == 3 and steps == 39 * (launched - 3) == 39 * 7
+    assert all(np.array_equal(x, y) for x, y in zip(s.get_state(), ref[:2]))
+    # a call of three loops waits at the first one's gate only
+    md.md_debug_loop(s.h, md.MD_HOLD_GATE)
+    s.step(5000)
+    assert md.md_debug_loop(s.h) == (launched + 3, steps, 4)
+    s.close()
