@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -62,6 +63,23 @@ bool within_allocation(const void* p, size_t bytes) {
     const CUdeviceptr at = (CUdeviceptr)(uintptr_t)p;
     return range && range(&base, &size, at) == CUDA_SUCCESS && at - base <= size && bytes <= size - (at - base);
 }
+
+// The md_step calls of this process that are under way on a device and could
+// run as one-launch loops (several handles, several threads): the sum of
+// 1024 / (loops of that size that fit the device at once).
+struct LoopDemand {
+    std::atomic<int>* sum = nullptr;
+    int mine = 0, total = 0;
+    void add(int device, int64_t blocks, int64_t fit) {
+        static std::atomic<int> of[64];
+        sum = &of[device & 63];
+        mine = (int)(1024 / (fit / blocks));
+        total = sum->fetch_add(mine) + mine;
+    }
+    ~LoopDemand() {
+        if (sum) sum->fetch_sub(mine);
+    }
+};
 
 // Zeroed storage for cudaGraphNodeParams (its union has no default
 // constructor).
@@ -801,9 +819,19 @@ struct Sim : SimBase {
         MD_CUDA(launch(kt.kickdrift, grid_atoms(), kBlock, a, nn));
         // After a loop that could not start, calls take graphs at once for a
         // while: a wait at the gate for each would cost more than the loops give.
-        const bool loops = run_rest == 0;
+        // So they do when the loops under way in other threads and this one
+        // ask for much more than the device has (kRunDemand).
+        bool loops = prm.use_graphs && !profiling && n > 1 && use_run();
+        LoopDemand demand;
+        if (loops) demand.add(device, run_grid(), run_blocks_max);
+        if (run_rest > 0) {
+            run_rest--;
+            loops = false;
+        } else if (loops && demand.total >= kRunDemand) {
+            run_rest = kRunDemandRest;
+            loops = false;
+        }
         const int64_t launched = loops_launched;
-        if (run_rest > 0) run_rest--;
         run_shut = false;
         int r = run_steps(n, loops);
         if (r) return r;

@@ -93,6 +93,14 @@ constexpr int kRunGatePolls = 1 << 12;         // polls before the gate gives up
 // Calls of md_step that take graphs at once after one whose loop did not start:
 // 1, then twice as many each time up to this, until a loop starts again.
 constexpr int kRunRestMax = 64;
+// Loops under way in several threads that fill the device kRunDemand / 1024
+// times or more give way to graphs for kRunDemandRest calls: loops that do not
+// fit at once take turns, where the handles' graphs interleave.  Calls of 100
+// steps, us per step of any handle, loops against graphs: 20011 atoms, 2 handles
+// (2.0 times) 6.97 and 8.89, 3 (3.0) 6.95 and 5.94, 4 (4.0) 6.94 and 4.63;
+// 9000 atoms, 8 handles (2.7) 2.28 and 2.55; 14000 atoms, 5 (2.5) 3.53 and 3.82.
+constexpr int kRunDemand = 3072;
+constexpr int kRunDemandRest = 16;
 // Elements per block of the cell-count scan (kBlock threads x 8).
 constexpr int kScanTile = 2048;
 // Largest neighbour capacity of the mixed form (its fixed-point partial

@@ -209,3 +209,39 @@ def test_a_loop_that_cannot_start_gives_way_to_graphs():
     s.step(5000)
     assert md.md_debug_loop(s.h) == (launched + 3, steps, 4)
     s.close()
+
+
+def test_many_large_loops_at_once_give_way_to_graphs():
+    # four loops of two thirds of the device each: calls that overlap take
+    # graphs, a handle alone its loops again after a while
+    n, k, calls = 20011, 100, 12
+    pos, vel, L = state(n, 0.8, 1.0, 57, jitter=0.05)
+    sims = [md.Simulation(L, n, RC, 0.4, DT) for _ in range(4)]
+    for s in sims:
+        s.set_state(pos, vel)
+    start = threading.Barrier(len(sims))
+
+    def work(s):
+        start.wait()
+        for _ in range(calls):
+            s.step(k)
+
+    threads = [threading.Thread(target=work, args=(s,)) for s in sims]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    launched = [md.md_debug_loop(s.h)[0] for s in sims]
+    assert sum(launched) < len(sims) * calls, launched
+    for _ in range(20):
+        sims[0].step(1 + k // 10)
+    assert md.md_debug_loop(sims[0].h)[0] > launched[0]
+    for _ in range(20):
+        sims[1].step(1 + k // 10)
+    out = [s.get_state() for s in sims]
+    assert all(np.array_equal(x, y) for x, y in zip(out[0], out[1]))
+    assert all(np.array_equal(x, y) for x, y in zip(out[2], out[3]))
+    for s in sims:
+        s.close()
+    ref = _run(pos, vel, L, [k] * calls, 0.4, use_graphs=False)
+    assert all(np.array_equal(x, y) for x, y in zip(out[2], ref[:2]))
