@@ -245,3 +245,23 @@ def test_many_large_loops_at_once_give_way_to_graphs():
         s.close()
     ref = _run(pos, vel, L, [k] * calls, 0.4, use_graphs=False)
     assert all(np.array_equal(x, y) for x, y in zip(out[2], ref[:2]))
+
+
+# which calls run in loops, by the steps that ran in them: sizes up to the last
+# that fits (about 12000 atoms without lists), the forms that have no loop
+@pytest.mark.parametrize("n,kw,loops", [
+    (29184, dict(), True), (29185, dict(), False), (500, dict(shell_bins=False), False),
+    (500, dict(precision="fp64"), False), (500, dict(build="warp"), False), (500, dict(variant="list_rows"), False),
+    (500, dict(use_graphs=False), False), (12000, dict(cell_list_only=True), True),
+    (12000, dict(cell_list_only=True, precision="fp64"), True), (30000, dict(cell_list_only=True), False)])
+def test_which_calls_run_in_loops(n, kw, loops):
+    pos, vel, L = state(n, 0.8, 1.0, 58, jitter=0.05)
+    s = md.Simulation(L, n, RC, 0.0 if "cell_list_only" in kw else 0.4, DT, **kw)
+    s.set_state(pos, vel)
+    for k in (1, 30, 2):
+        s.step(k)
+    assert md.md_debug_loop(s.h) == ((2, 30, 0) if loops else (0, 0, 0))
+    s.set_profiling(True)
+    s.step(3)
+    assert md.md_debug_loop(s.h)[0] == (2 if loops else 0)
+    s.close()
