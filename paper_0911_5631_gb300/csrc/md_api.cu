@@ -692,8 +692,8 @@ struct Sim : SimBase {
         return rebuild_eager();
     }
 
-    // loops: as in run_steps
-    int finish_pending(int64_t* steps_left_out, bool loops) {
+    // asked: steps queued; loops: as in run_steps
+    int finish_pending(int64_t* steps_left_out, int64_t asked, bool loops) {
         bool overflowed = false;
         // a loop that other work on the GPU kept from starting as a whole has
         // done nothing: the rest of this call runs as graphs
@@ -734,10 +734,12 @@ struct Sim : SimBase {
             }
             if (c.steps_left > 0 && c.error == 0) {
                 // steps that waited for a rebuild inside a graph: run them
-                // now (each round leaves fewer to wait; the last few take
-                // graphs of one step, which never wait)
-                r = run_steps(c.steps_left, loops, c.steps_left < kChunks[0]);
+                // now (each round leaves fewer to wait; the last few of a
+                // system in which most steps wait take graphs of one step,
+                // which never do)
+                r = run_steps(c.steps_left, loops, c.steps_left < kChunks[0] && 2 * c.steps_left > asked);
                 if (r) return r;
+                asked = c.steps_left;
                 continue;
             }
             if (steps_left_out) *steps_left_out = c.steps_left;
@@ -836,7 +838,7 @@ struct Sim : SimBase {
         int r = run_steps(n, loops);
         if (r) return r;
         int64_t left = 0;
-        r = finish_pending(&left, loops);
+        r = finish_pending(&left, n, loops);
         if (r) return r;
         if (run_shut) run_rest = run_backoff = run_backoff ? std::min(2 * run_backoff, kRunRestMax) : 1;
         else if (loops_launched != launched) run_backoff = 0;
