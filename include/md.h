@@ -282,8 +282,9 @@ const char* md_last_error(const md_handle* h);
 /* Device self-check of the library's integer-pipe number conversions
  * (binary32<->binary64, binary32<->int64 fixed point) against the hardware
  * conversions on n hashed inputs (uses the current device).  failures[0..3]
- * receive the mismatch counts for float->double, double->float,
- * float->int64 and int64->float.  MD_ENODEV without a GPU. */
+ * receive the mismatch counts for float->double, double->float (and
+ * reciprocals of the FP64 pair term more than one unit in the last place from
+ * the quotient), float->int64 and int64->float.  MD_ENODEV without a GPU. */
 int md_selftest(int64_t n, int64_t failures[4]);
 
 /* ---- forces without device allocation --------------------------------

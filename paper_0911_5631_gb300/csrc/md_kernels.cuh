@@ -397,19 +397,6 @@ struct Fix2 {
     }
 };
 
-// 1 / a.  The seed (rcp.approx.ftz.f64, good to about 2^-20) is refined by
-// one third-order step of Householder's iteration for the reciprocal,
-// y (1 + e + e^2) with e = 1 - a y, whose error e^3 is below 2^-53: three
-// FP64 operations where the division takes about ten.  An infinite seed
-// (a = 0) is the result.
-__device__ __forceinline__ double reciprocal(double a) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double e = fma(-a, y, 1.0);
-    const double r = fma(y, fma(e, e, e), y);
-    return (__double2hiint(y) & 0x7fffffff) == 0x7ff00000 ? y : r;
-}
-
 // a < b for non-negative doubles, compared as integers: a comparison on the
 // FP64 pipe costs as much as an addition.  A NaN of either sign counts as
 // large (the hardware's own has its sign bit set).
@@ -2506,7 +2493,8 @@ __global__ void __launch_bounds__(kBlock) k_get_cells(Args<P> a, int* out) {
 
 // Compares the FP32/integer-pipe conversions with the hardware conversions
 // on hashed bit patterns spanning the magnitudes the step uses.  fails[k]
-// counts mismatches of f64, f32, the fixed-point accumulation and from_fix.
+// counts mismatches of f64, f32 (and the reciprocal), the fixed-point
+// accumulation and from_fix.
 __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
     z += 0x9E3779B97F4A7C15ull;
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -2528,6 +2516,11 @@ __global__ void __launch_bounds__(kBlock) k_selftest(long long n, unsigned long 
     unsigned long long e64 = 1023ull - 120ull + (r2 % 240ull);
     double d = __longlong_as_double((long long)((r2 & 0x800FFFFFFFFFFFFFull) | (e64 << 52)));
     if (__float_as_uint(cvt::f32(d)) != __float_as_uint(__double2float_rn(d))) atomicAdd(&fails[1], 1ull);
+    // the FP64 pair term's reciprocal: e^3 and the rounding of e + e^2 are below
+    // 2^-5 ulp, the last operation's rounding is half an ulp, and the quotient's
+    // own another, so the two are neighbours at most
+    long long apart = __double_as_longlong(reciprocal(fabs(d))) - __double_as_longlong(1.0 / fabs(d));
+    if (apart < -1 || apart > 1) atomicAdd(&fails[1], 1ull);
     // fixed point: g with |g| in [2^-40, 2^30); g and -g cancel exactly
     float g = __uint_as_float((unsigned)((r >> 16) & 0x807FFFFFu) | ((87u + (unsigned)(r2 % 70u)) << 23));
     Fix one, both;

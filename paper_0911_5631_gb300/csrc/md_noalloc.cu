@@ -20,6 +20,7 @@
 #include <string>
 
 #include "../../include/md.h"
+#include "md_common.cuh"
 
 namespace md {
 // Records the message md_last_error(NULL) returns (defined with the rest of
@@ -293,19 +294,6 @@ __global__ void __launch_bounds__(1024) nz_bin_small(Geo g, Scratch s, const dou
     for (int k = tid; k < g.n; k += 1024) place_atom(g, s, pos, s_order[k], k);
 }
 
-// 1 / a.  The seed (rcp.approx.ftz.f64, good to about 2^-20) is refined by
-// one third-order step of Householder's iteration for the reciprocal,
-// y (1 + e + e^2) with e = 1 - a y, whose error e^3 is below 2^-53: three
-// FP64 operations where the division takes about ten.  An infinite seed
-// (a = 0) is the result.
-__device__ __forceinline__ double reciprocal(double a) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double e = fma(-a, y, 1.0);
-    const double r = fma(y, fma(e, e, e), y);
-    return (__double2hiint(y) & 0x7fffffff) == 0x7ff00000 ? y : r;
-}
-
 // Forces on every atom from the 27 cells around its cell, and the sums of
 // 1/2 sum_j u and 1/2 sum_j r.f (each pair is seen from both atoms).
 //
@@ -359,7 +347,7 @@ __global__ void __launch_bounds__(kThreads, 4) nz_force(Geo g, Scratch s, double
             if (z < 0 || z >= g.G[2]) ez += z < 0 ? g.L[2] : -g.L[2];
             const double r2 = fma(ez, ez, fma(ey, ey, ex * ex));
             if (r2 < g.rc2) {
-                const double ir2 = reciprocal(r2);
+                const double ir2 = md::reciprocal(r2);
                 const double ir6 = ir2 * ir2 * ir2;
                 const double fr = fma(48.0, ir6, -24.0) * ir6 * ir2;
                 fx = fma(fr, ex, fx);
