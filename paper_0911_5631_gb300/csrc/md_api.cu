@@ -504,9 +504,11 @@ struct Sim : SimBase {
     // Whether plain steps run in a one-launch loop of md_run.cuh: the
     // cell-list-only variant, or the mixed form with sorted lists and the
     // default kernels, and a system whose blocks are all resident at once
-    // (about 12000 and 29184 atoms).  It wins wherever
-    // it applies: 100 steps and their read-back take 0.66 ms instead of 1.77
-    // at 2048 atoms and 1.15 ms instead of 2.05 at 20011.
+    // (about 12000 and 29184 atoms).  Alone on the device it wins over that
+    // range: 100 steps of 2048, 20011 and 29184 atoms take 0.46, 0.74 and
+    // 0.80 ms, in graphs 1.43, 1.62 and 1.67; cells only, 12000 atoms, 2.1
+    // (mixed) and 3.0 ms (FP64) against 5.7 and 15.7; two steps, of which one
+    // runs in the loop, 57 us against 60 (2048) and 58 against 68 (29184).
     bool use_run() {
         if (run_threads() == 0) return false;
         if (run_blocks_max < 0) {
