@@ -666,8 +666,6 @@ struct Sim : SimBase {
             return MD_ECUDA;
         }
         if (c.error & (kErrUnstable | kErrClose)) {
-            // (a non-finite input is binned at its cell's centre, where it may
-            // meet another)
             err = (c.error & kErrUnstable) ? "non-finite coordinate or velocity"
                                            : "two atoms came closer than the fixed-point force range allows";
             return MD_EUNSTABLE;
@@ -791,8 +789,8 @@ struct Sim : SimBase {
         MD_CUDA(launch(kt.set_state, grid_atoms(), kBlock, in));
         int r = rebuild_eager();
         if (r) return r;
-        // the forces follow at once; a list that turns out to have overflowed
-        // is grown and they are computed again
+        // the forces follow at once, unless the list has overflowed: the kernel
+        // then does nothing, the list is grown and it is launched again
         for (int attempt = 0; attempt < 8; attempt++) {
             r = step_kernel_eager(kModeInit, true);
             if (r) return r;

@@ -2288,7 +2288,9 @@ __global__ void __launch_bounds__(kB, P::kFp64 ? (kB == kBlock ? 3 : 5) : 5 * kB
     // a step whose rebuild is due but has not run (a graph checks for
     // rebuilds every kRebuildEvery steps) waits: it does nothing, and the
     // call runs one step more at its end
-    const bool active = init || (err == 0 && left > 0 && !misplaced && !vw.pend);
+    // (nor does the load's evaluation of a list that overflowed: `lim` counts
+    // entries that its columns do not hold)
+    const bool active = err == 0 && (init || (left > 0 && !misplaced && !vw.pend));
     const bool energy = init || last;
     const pos4* pc = par ? a.pB : a.pA;
     pos4* pn = par ? a.pA : a.pB;
@@ -2383,7 +2385,7 @@ __global__ void k_step_tail(Args<P> a, int mode, cudaGraphConditionalHandle next
     const bool init = kFinal && (mode == kModeInit);
     const bool last = kFinal && !init && in.left == 1;
     const bool misplaced = !kFinal && in.left == 1;
-    const bool active = init || (in.err == 0 && in.left > 0 && !misplaced && !in.pend);
+    const bool active = in.err == 0 && (init || (in.left > 0 && !misplaced && !in.pend));
     close_step<P>(a, in, d2, in.err, in.left, in.par, init, last, misplaced, active, next, has_next);
 }
 

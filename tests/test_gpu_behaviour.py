@@ -295,3 +295,28 @@ def test_a_device_array_that_is_too_short_is_refused():
     s.set_state(pos, vel)
     s.step(10)
     s.close()
+
+
+# a capacity below the first build's lists: the load grows them, and its forces
+# are those of lists that were large enough (sorted lists, whose counts per
+# shell bin exceed the capacity before they have grown, and direct ones)
+@pytest.mark.parametrize("kw", [dict(), dict(variant="list_rows"), dict(variant="plain_loads"), dict(variant="block256"),
+                                dict(shell_bins=False), dict(build="warp"), dict(precision="fp64"), dict(rc=2.5)])
+@pytest.mark.parametrize("n", [500, 2048, 2916])
+def test_loading_more_neighbours_than_the_capacity(n, kw):
+    kw = dict(kw)
+    rc = kw.pop("rc", RC)
+    pos, vel, L = state(n, 0.95, 1.0, 17)
+    out = []
+    for cap in (8, 0):
+        s = md.Simulation(L, n, rc, 0.1, DT, nbr_capacity=cap, **kw)
+        s.set_state(pos, vel)
+        assert s.plan()["nbr_capacity"] > 8
+        out.append((s.forces(), s.measure()["pe"]))
+        s.step(5)
+        out[-1] += s.get_state()
+        s.close()
+    if kw.get("precision") == "fp64":  # (the order of the lists may differ)
+        assert np.abs(out[0][0] - out[1][0]).max() <= 1e-11 * max(1.0, np.abs(out[1][0]).max())
+    else:
+        assert all(np.array_equal(x, y) for x, y in zip(out[0], out[1]))
