@@ -674,6 +674,14 @@ template <> struct AccOf<F64> { using type = AccF64; };
 // 1M atoms, most of a warp's lanes idle at each FP64 instruction; this takes
 // 250 us, with the FP64 pipe 82 % busy.
 //
+// Where the queues are about equally long (lists with many interacting
+// entries) or a round's additions cost more than idle lanes (the energy step,
+// whose five sums leave a window of 32 terms that three or so lanes add up one
+// after the other), each lane evaluates its own queue: the same operations in
+// the same order, so the same bits.  Numbered throughout, the energy step of 1M
+// atoms took 0.54 ms for soft spheres and 9.1 ms with r_c = 2.5 (0.45 and 3.8
+// now; 4.7 when every lane tested in FP64), and 33 steps 110 ms (99; 130).
+//
 // rows: the warp's staged rows (kStageRows x 32 ints); tab: 9 x 32 doubles;
 // res: kRes x (3, or 5 with kEnergy) doubles.  Every lane of the warp must
 // call it (cnt = 0 for a lane without an atom).
@@ -692,6 +700,34 @@ __device__ __forceinline__ void forces_fp64(const Args<F64>& a, int cnt, const i
         tab[(3 + k) * 32 + lane] = k == 0 ? __dadd_rn(qy, a.w[1]) : (k == 1 ? qy : __dsub_rn(qy, a.w[1]));
         tab[(6 + k) * 32 + lane] = k == 0 ? __dadd_rn(qz, a.w[2]) : (k == 1 ? qz : __dsub_rn(qz, a.w[2]));
     }
+    constexpr int kSums = kEnergy ? 5 : 3;
+    // the terms of entry e of the atom in lane `own`, each rounded by itself
+    // (zero outside r_c)
+    auto terms = [&](unsigned e, int own, double (&g)[5]) {
+        const double2* pj = reinterpret_cast<const double2*>(pc + (e & jmask));
+        const double2 pxy = __ldg(pj);
+        const double pz = __ldg(reinterpret_cast<const double*>(pj + 1));
+        const unsigned c = e >> kCodeShift;
+        const double dx = tab[(c & 3u) * 32 + own] - pxy.x;
+        const double dy = tab[(3 + ((c >> 2) & 3u)) * 32 + own] - pxy.y;
+        const double dz = tab[(6 + (c >> 4)) * 32 + own] - pz;
+        const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+#pragma unroll
+        for (int k = 0; k < 5; k++) g[k] = 0.0;
+        if (less_bits(r2, a.rc2)) {
+            acc.close |= less_bits(r2, a.close2);
+            const double ir2 = reciprocal(r2);
+            const double ir6 = ir2 * ir2 * ir2;
+            const double fr = fma(48.0, ir6, -24.0) * ir6 * ir2;
+            g[0] = __dmul_rn(fr, dx);
+            g[1] = __dmul_rn(fr, dy);
+            g[2] = __dmul_rn(fr, dz);
+            if constexpr (kEnergy) {
+                g[3] = fma(fma(4.0, ir6, -4.0), ir6, a.ushift);
+                g[4] = __dmul_rn(fr, r2);
+            }
+        }
+    };
     int nq = 0;
     auto flush = [&]() {
         int incl = nq;
@@ -701,6 +737,26 @@ __device__ __forceinline__ void forces_fp64(const Args<F64>& a, int cnt, const i
             if (lane >= o) incl += y;
         }
         const int excl = incl - nq, total = __shfl_sync(kFull, incl, 31);
+        const int most = __reduce_max_sync(kFull, nq);
+        // FP64 instructions of the two ways: each lane through its own queue, or
+        // numbered, when a window of kRes terms costs its lanes' additions one
+        // after the other
+        if (most * (17 + kSums) < 17 * ((total + 31) / 32) + kSums * most * ((total + kRes - 1) / kRes)) {
+            for (int q = 0; q < nq; q++) {
+                double g[5];
+                terms((unsigned)rows[q * 32 + lane], lane, g);
+                acc.fx = __dadd_rn(acc.fx, g[0]);
+                acc.fy = __dadd_rn(acc.fy, g[1]);
+                acc.fz = __dadd_rn(acc.fz, g[2]);
+                if constexpr (kEnergy) {
+                    acc.u = __dadd_rn(acc.u, g[3]);
+                    acc.w = __dadd_rn(acc.w, g[4]);
+                }
+            }
+            __syncwarp();
+            nq = 0;
+            return;
+        }
         __syncwarp();
         for (int base = 0; base < total; base += kRes) {
             const int top = min(total - base, kRes);
@@ -713,31 +769,10 @@ __device__ __forceinline__ void forces_fp64(const Args<F64>& a, int cnt, const i
                 own = min(own, 31);
                 const int first = __shfl_sync(kFull, excl, own);
                 if (r + lane >= top) continue;
-                const unsigned e = (unsigned)rows[(p - first) * 32 + own];
-                const double2* pj = reinterpret_cast<const double2*>(pc + (e & jmask));
-                const double2 pxy = __ldg(pj);
-                const double pz = __ldg(reinterpret_cast<const double*>(pj + 1));
-                const unsigned c = e >> kCodeShift;
-                const double dx = tab[(c & 3u) * 32 + own] - pxy.x;
-                const double dy = tab[(3 + ((c >> 2) & 3u)) * 32 + own] - pxy.y;
-                const double dz = tab[(6 + (c >> 4)) * 32 + own] - pz;
-                const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-                double g[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-                if (less_bits(r2, a.rc2)) {
-                    acc.close |= less_bits(r2, a.close2);
-                    const double ir2 = reciprocal(r2);
-                    const double ir6 = ir2 * ir2 * ir2;
-                    const double fr = fma(48.0, ir6, -24.0) * ir6 * ir2;
-                    g[0] = fr * dx;
-                    g[1] = fr * dy;
-                    g[2] = fr * dz;
-                    if constexpr (kEnergy) {
-                        g[3] = fma(fma(4.0, ir6, -4.0), ir6, a.ushift);
-                        g[4] = fr * r2;
-                    }
-                }
+                double g[5];
+                terms((unsigned)rows[(p - first) * 32 + own], own, g);
 #pragma unroll
-                for (int k = 0; k < (kEnergy ? 5 : 3); k++) res[k * kRes + r + lane] = g[k];
+                for (int k = 0; k < kSums; k++) res[k * kRes + r + lane] = g[k];
             }
             __syncwarp();
             const int t1 = min(excl + nq - base, top);
@@ -2117,9 +2152,9 @@ __device__ __forceinline__ void stage_wait() {
     }
 }
 
-// Terms a warp of the FP64 list form holds at a time: the warp's survivors of
-// most fluids in the plain step; one round in the final step, whose five sums
-// and 256-thread blocks leave less shared memory.
+// Terms a warp of the FP64 list form holds at a time when it numbers them: the
+// warp's survivors of most fluids in the plain step; one round in the final
+// step, whose five sums and 256-thread blocks leave less shared memory.
 __host__ __device__ constexpr int f64_results(bool final_step) { return final_step ? 32 : 160; }
 
 // The per-atom part of a step (Sec. 3.1 (c)-(e) and (a) of the next step):
