@@ -678,9 +678,10 @@ template <> struct AccOf<F64> { using type = AccF64; };
 // entries) or a round's additions cost more than idle lanes (the energy step,
 // whose five sums leave a window of 32 terms that three or so lanes add up one
 // after the other), each lane evaluates its own queue: the same operations in
-// the same order, so the same bits.  Numbered throughout, the energy step of 1M
-// atoms took 0.54 ms for soft spheres and 9.1 ms with r_c = 2.5 (0.45 and 3.8
-// now; 4.7 when every lane tested in FP64), and 33 steps 110 ms (99; 130).
+// the same order, so the same bits.  Numbered throughout, md_step(1), an energy
+// step, took 119 us for 130000 soft spheres and 9.2 ms for 1M atoms with
+// r_c = 2.5 (106 us and 3.8 ms now; 129 us and 4.7 ms when every lane tested in
+// FP64), and 33 steps of the latter 110 ms (99; 130).
 //
 // rows: the warp's staged rows (kStageRows x 32 ints); tab: 9 x 32 doubles;
 // res: kRes x (3, or 5 with kEnergy) doubles.  Every lane of the warp must
@@ -1313,29 +1314,30 @@ __device__ __forceinline__ bool sorts_cells(int reorder) {
     return P::kFp64 || reorder;
 }
 
-// The candidate that an atom is to the neighbour search: its FP32 coordinates
-// in its cell and its storage index.  Right after a binning the displacement
-// is what FP32 left of the offset (or 0), so pb is the coordinate.
-template <class P>
-__device__ __forceinline__ float4 candidate(const Args<P>& a, int64_t i, int index) {
-    return make_float4(to_f32(a.pbx[i]), to_f32(a.pby[i]), to_f32(a.pbz[i]), __int_as_float(index));
+// The candidate that an atom is to the neighbour search (and, in the mixed
+// cells-only variant, to the forces): its pair coordinate, which the binning has
+// just written, and its storage index.  (pb alone is the same number but for an
+// offset that FP32 rounds onto half a unit of pb's last place.)
+__device__ __forceinline__ float4 candidate(const Args<Mixed>& a, int64_t i, int index, int parity) {
+    const float4 p = (parity ? a.pB : a.pA)[i];
+    return make_float4(p.x, p.y, p.z, __int_as_float(index));
 }
 
 // Places each atom at cell_start[cell] + rank (the cell's arrival order).
 template <class P>
-__device__ __forceinline__ void scatter_item(const Args<P>& a, int64_t t, int reorder) {
+__device__ __forceinline__ void scatter_item(const Args<P>& a, int64_t t, int reorder, int parity) {
     const int slot = a.cell_start[cell_index_of_packed(a.cell[t], a.G)] + a.rank[t];
     if (slot < 0 || slot >= a.n) atomicOr(&a.ctr->error, kErrUnstable);
     else if (sorts_cells<P>(reorder)) a.order[slot] = (int)t;
-    else a.cand[slot] = candidate(a, t, (int)t);
+    else if constexpr (!P::kFp64) a.cand[slot] = candidate(a, t, (int)t, parity);
 }
 
 // ... and clears the counts for the next binning.
 template <class P>
 __global__ void __launch_bounds__(kBlock) k_scatter(Args<P> a, int guard) {
     if (guard && !a.ctr->rebuild_flag) return;
-    const int reorder = a.ctr->reorder_now;
-    for (int64_t t = gtid(); t < a.n; t += (int64_t)gridDim.x * blockDim.x) scatter_item<P>(a, t, reorder);
+    const int reorder = a.ctr->reorder_now, parity = a.ctr->parity;
+    for (int64_t t = gtid(); t < a.n; t += (int64_t)gridDim.x * blockDim.x) scatter_item<P>(a, t, reorder, parity);
     // counts and tile totals are no longer needed once cell_start is known
     for (int64_t t = gtid(); t < a.ncells; t += (int64_t)gridDim.x * blockDim.x) a.count[t] = 0;
     for (int64_t t = gtid(); t < a.ntiles; t += (int64_t)gridDim.x * blockDim.x) a.tile_sum[t] = 0;
@@ -1384,12 +1386,20 @@ __device__ __forceinline__ void cellsort_item(const Args<P>& a, int64_t c) {
 template <class P>
 __device__ __forceinline__ void gather_item(const Args<P>& a, int64_t s, int reorder) {
     const int i = a.order[s];
-    a.cand[s] = candidate(a, i, reorder ? (int)s : i);
+    const auto pbx = a.pbx[i], pby = a.pby[i], pbz = a.pbz[i];
+    double ox = 0.0, oy = 0.0, oz = 0.0;
+    if (!P::kFp64 || reorder) {  // (FP64: no displacement right after a binning)
+        ox = a.ox[i];
+        oy = a.oy[i];
+        oz = a.oz[i];
+    }
+    a.cand[s] = make_float4(to_f32(pair_coord(pbx, ox)), to_f32(pair_coord(pby, oy)), to_f32(pair_coord(pbz, oz)),
+                            __int_as_float(reorder ? (int)s : i));
     if (reorder) {
         a.s_cell[s] = a.cell[i];
         a.s_perm[s] = a.perm[i];
-        a.s_pbx[s] = a.pbx[i]; a.s_pby[s] = a.pby[i]; a.s_pbz[s] = a.pbz[i];
-        a.s_ox[s] = a.ox[i]; a.s_oy[s] = a.oy[i]; a.s_oz[s] = a.oz[i];
+        a.s_pbx[s] = pbx; a.s_pby[s] = pby; a.s_pbz[s] = pbz;
+        a.s_ox[s] = ox; a.s_oy[s] = oy; a.s_oz[s] = oz;
         a.s_vx[s] = a.vx[i]; a.s_vy[s] = a.vy[i]; a.s_vz[s] = a.vz[i];
     }
 }
@@ -2696,8 +2706,8 @@ __device__ __noinline__ void ens_rebuild(const Args<P>& a, EnsShared& sh, int* s
     tm.sync();
     if (tm.lead_block()) ens_scan<P>(a, sh);
     tm.sync();
-    const int reorder = C->reorder_now;
-    for (int64_t t = t0; t < n; t += dt) scatter_item<P>(a, t, reorder);
+    const int reorder = C->reorder_now, parity = C->parity;
+    for (int64_t t = t0; t < n; t += dt) scatter_item<P>(a, t, reorder, parity);
     for (int64_t c = t0; c < a.ncells; c += dt) a.count[c] = 0;
     tm.sync();
     if (reorder) {
@@ -2705,7 +2715,7 @@ __device__ __noinline__ void ens_rebuild(const Args<P>& a, EnsShared& sh, int* s
         tm.sync();
         for (int64_t s = t0; s < n; s += dt) gather_item<P>(a, s, reorder);
         tm.sync();
-        for (int64_t s = t0; s < n; s += dt) commit_item<P>(a, s, C->parity);
+        for (int64_t s = t0; s < n; s += dt) commit_item<P>(a, s, parity);
         tm.sync();
     }
     int mx = 0;

@@ -366,7 +366,7 @@ __device__ __noinline__ int run_rebuild(const Args<P>& a, int64_t i, int par, in
     said = bar.sync(0, s_sync, C);
     if (said & kRunStop) return said;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, dt = (int64_t)gridDim.x * blockDim.x;
-    if (in && sub == 0) scatter_item<P>(a, i, reorder);
+    if (in && sub == 0) scatter_item<P>(a, i, reorder, par);
     for (int64_t c = t0; c < a.ncells; c += dt) a.count[c] = 0;
     for (int64_t c = t0; c < a.ntiles; c += dt) a.tile_sum[c] = 0;
     said = bar.sync(0, s_sync, C);
@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(kRunCellBlock, 5) k_run_cells(Args<P> a, long 
         if (bar.sync(0, &s_sync, C) & kRunStop) break;
         for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) run_scan_tile(a, t, s_scan);
         if (bar.sync(0, &s_sync, C) & kRunStop) break;
-        if (t0 < a.n) scatter_item<P>(a, t0, reorder);
+        if (t0 < a.n) scatter_item<P>(a, t0, reorder, par);
         for (int64_t c = t0; c < a.ncells; c += dt) a.count[c] = 0;
         for (int64_t c = t0; c < a.ntiles; c += dt) a.tile_sum[c] = 0;
         if (bar.sync(0, &s_sync, C) & kRunStop) break;
