@@ -1387,14 +1387,21 @@ template <class P>
 __device__ __forceinline__ void gather_item(const Args<P>& a, int64_t s, int reorder) {
     const int i = a.order[s];
     const auto pbx = a.pbx[i], pby = a.pby[i], pbz = a.pbz[i];
-    double ox = 0.0, oy = 0.0, oz = 0.0;
-    if (!P::kFp64 || reorder) {  // (FP64: no displacement right after a binning)
+    const int index = reorder ? (int)s : i;
+    double ox, oy, oz;
+    if constexpr (P::kFp64) {  // right after a binning the displacement is 0
+        a.cand[s] = make_float4(to_f32(pbx), to_f32(pby), to_f32(pbz), __int_as_float(index));
+        if (reorder) {
+            ox = a.ox[i];
+            oy = a.oy[i];
+            oz = a.oz[i];
+        }
+    } else {
         ox = a.ox[i];
         oy = a.oy[i];
         oz = a.oz[i];
+        a.cand[s] = make_float4(pair_coord(pbx, ox), pair_coord(pby, oy), pair_coord(pbz, oz), __int_as_float(index));
     }
-    a.cand[s] = make_float4(to_f32(pair_coord(pbx, ox)), to_f32(pair_coord(pby, oy)), to_f32(pair_coord(pbz, oz)),
-                            __int_as_float(reorder ? (int)s : i));
     if (reorder) {
         a.s_cell[s] = a.cell[i];
         a.s_perm[s] = a.perm[i];

@@ -501,3 +501,28 @@ def test_rescale_rejects_bad_temperature():
             s.rescale(T)
         assert e.value.code == md.MD_EINVAL
     s.close()
+
+
+def test_cells_only_forces_take_the_pair_coordinate():
+    # an offset in its cell whose FP32 value and the rest of it, rounded to
+    # FP32, add up to the next number: the pair coordinate that the list form
+    # uses.  A pair along x has the same operations in both variants
+    L, rc = np.array([4.6, 4.6, 4.6]), RC  # four cells along an edge in both
+    w = L[0] / 4
+    centre = 2.5 * w - 0.5 * L[0]
+    pb = np.nextafter(np.float32(0.3), np.float32(1.0))
+    if pb.view(np.uint32) % 2 == 0:
+        pb = np.nextafter(pb, np.float32(1.0))
+    x = centre + (float(pb) + 2.0 ** -26 - 2.0 ** -53)
+    t = x - centre
+    o = t - float(np.float32(t))
+    assert np.float32(t) == pb and pb + np.float32(o) != pb
+    for d in (0.95, 1.0, 1.05):
+        pos = np.array([[x, 0.1, 0.1], [x - d, 0.1, 0.1]])
+        f = []
+        for kw in (dict(skin=0.02), dict(skin=0.0, cell_list_only=True)):
+            s = sim(pos, np.zeros((2, 3)), L, **kw)
+            assert list(s.plan()["G"]) == [4, 4, 4]
+            f.append(s.forces())
+            s.close()
+        assert f[0][0, 0] != 0.0 and np.array_equal(f[0], f[1])
