@@ -43,6 +43,19 @@ thread_local std::string g_create_error;
 // the energy kernel.
 constexpr int kChunks[] = {10 * kRebuildEvery, kRebuildEvery, 1};
 constexpr int kNumChunks = sizeof(kChunks) / sizeof(kChunks[0]);
+// A call may also end in a graph of kTail steps whose last is that step, where
+// that makes fewer graphs: 32 and 33 steps of 130000 atoms took 540 and 566 us
+// in graphs of 30 and 1, 531 and 561 with it.
+constexpr int kTail = 32;
+// graphs that n plain steps take
+constexpr int64_t chunks_of(int64_t n) {
+    int64_t c = 0;
+    for (int k : kChunks) {
+        c += n / k;
+        n %= k;
+    }
+    return c;
+}
 
 // Whether the `bytes` bytes at device address p lie within one allocation
 // (what a copy checks of its arguments, and a kernel does not).
@@ -151,7 +164,7 @@ struct Sim : SimBase {
         cudaGraph_t g = nullptr;
         cudaGraphExec_t e = nullptr;
     };
-    Chunk plain[kNumChunks], last;  // instantiated when first used
+    Chunk plain[kNumChunks], last, tail;  // instantiated when first used
 
     bool profiling = false;
     std::vector<cudaEvent_t> ev;
@@ -391,6 +404,7 @@ struct Sim : SimBase {
     void destroy_graphs() {
         for (Chunk& c : plain) destroy_graph(c);
         destroy_graph(last);
+        destroy_graph(tail);
     }
 
     template <class... T>
@@ -429,8 +443,8 @@ struct Sim : SimBase {
         return MD_OK;
     }
 
-    // K steps, plain ones or (final_node, K = 1) the one that may be a call's
-    // last: k_cond, then per step the step kernel and its closing kernel,
+    // K steps, plain ones or (final_node) with the one that may be a call's
+    // last at their end: k_cond, then per step the step kernel and its closing kernel,
     // with a conditional rebuild node before every m-th step.  The
     // cell-list-only form rebuilds at every step: its graphs hold the
     // rebuild's kernels themselves (a conditional node costs about 5 us), each
@@ -450,10 +464,11 @@ struct Sim : SimBase {
         }
         int mode = kModeAuto;
         for (int s = 0; s < K; s++) {
+            const bool fin = final_node && s + 1 == K;
             if (prm.cell_list_only) {
                 int r = add_rebuild(c.g, &prev, 1);
                 if (r) return r;
-                MD_CUDA(add_kernel(c.g, &prev, &node, cells_fn(final_node), cells_grid(), kBlock, a));
+                MD_CUDA(add_kernel(c.g, &prev, &node, cells_fn(fin), cells_grid(), kBlock, a));
                 prev = node;
             } else if (s % m == 0) {
                 NodeParams buf;
@@ -471,11 +486,10 @@ struct Sim : SimBase {
             }
             const int has = (!prm.cell_list_only && s + 1 < K && (s + 1) % m == 0) ? 1 : 0;
             cudaGraphConditionalHandle nxt = has ? h[(s + 1) / m] : 0;
-            MD_CUDA(add_kernel(c.g, &prev, &node, step_fn(final_node), step_grid(final_node), step_block(final_node),
-                               a, mode, nxt, has));
+            MD_CUDA(add_kernel(c.g, &prev, &node, step_fn(fin), step_grid(fin), step_block(fin), a, mode, nxt, has));
             if (kStepTailNode) {
                 cudaGraphNode_t stepn = node;
-                MD_CUDA(add_kernel(c.g, &stepn, &node, tail_fn(final_node), 1, 32, a, mode, nxt, has));
+                MD_CUDA(add_kernel(c.g, &stepn, &node, tail_fn(fin), 1, 32, a, mode, nxt, has));
             }
             prev = node;
         }
@@ -574,12 +588,14 @@ struct Sim : SimBase {
                 if (r) return r;
                 left = 0;
             }
+            const bool with_tail = !single && left + 1 >= kTail && chunks_of(left + 1 - kTail) < chunks_of(left);
+            if (with_tail) left -= kTail - 1;
             for (int k = single ? kNumChunks - 1 : 0; k < kNumChunks; k++) {
                 int r = replay(plain[k], kChunks[k], false, left / kChunks[k]);
                 if (r) return r;
                 left %= kChunks[k];
             }
-            int r = replay(last, 1, true, 1);
+            int r = with_tail ? replay(tail, kTail, true, 1) : replay(last, 1, true, 1);
             if (r) return r;
         } else {
             if (profiling && (int64_t)ev.size() < 4 * nsteps) {

@@ -320,3 +320,24 @@ def test_loading_more_neighbours_than_the_capacity(n, kw):
         assert np.abs(out[0][0] - out[1][0]).max() <= 1e-11 * max(1.0, np.abs(out[1][0]).max())
     else:
         assert all(np.array_equal(x, y) for x, y in zip(out[0], out[1]))
+
+
+# counts around the lengths of the graphs, each against stream launches: a call
+# that ends in the graph of 32 steps, in one of its own, and with what is left
+@pytest.mark.parametrize("n,kw", [(500, dict(shell_bins=False)), (500, dict(precision="fp64")),
+                                  (14000, dict(skin=0.0, cell_list_only=True))])
+def test_graph_lengths(n, kw):
+    kw = dict(kw)
+    skin = kw.pop("skin", 0.2)
+    pos, vel, L = state(n, 0.8, 2.0, 18, jitter=0.05)
+    steps = (31, 32, 33, 34, 64, 65, 30, 96, 128, 2)
+    out = []
+    for graphs in (True, False):
+        s = sim(pos, vel, L, skin=skin, use_graphs=graphs, **kw)
+        for k in steps:
+            s.step(k)
+            out.append(s.get_state() + (s.measure(),))
+        s.close()
+    for a, b in zip(out[:len(steps)], out[len(steps):]):
+        assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+        assert all(a[2][k] == b[2][k] for k in ("step", "rebuilds", "reorders", "ke", "pe", "virial"))
