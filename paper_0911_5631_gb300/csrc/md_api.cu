@@ -389,8 +389,14 @@ struct Sim : SimBase {
         return MD_OK;
     }
     // the cell-list-only variant's force kernel, run before its step kernel
-    void* cells_fn(bool final_node) const { return final_node ? kt.cell_forces_final : kt.cell_forces; }
-    unsigned cells_grid() const { return (unsigned)((a.n * kCellLanes + kBlock - 1) / kBlock); }
+    bool cells_wide() const { return !P::kFp64 && a.n >= kCellWide; }
+    void* cells_fn(bool final_node) const {
+        if (cells_wide()) return final_node ? kt.cell_forces_wide_final : kt.cell_forces_wide;
+        return final_node ? kt.cell_forces_final : kt.cell_forces;
+    }
+    unsigned cells_grid() const {
+        return (unsigned)((a.n * (cells_wide() ? 1 : kCellLanes) + kBlock - 1) / kBlock);
+    }
     void* tail_fn(bool final_node) const { return final_node ? kt.step_tail_final : kt.step_tail; }
 
     // ---- graphs ----------------------------------------------------------

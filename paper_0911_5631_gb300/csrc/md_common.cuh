@@ -75,6 +75,11 @@ static_assert(kEnsBuildStage < 256, "one byte per shell bin in a 64-bit word");
 constexpr int kEnsSmemInts = kStageRows > 2 * kEnsBuildStage ? kStageRows : 2 * kEnsBuildStage;
 // Lanes that share an atom in the force kernel of the cell-list-only variant.
 constexpr int kCellLanes = 8;
+// Atoms from which the mixed form takes a thread per atom there.  us per
+// step with eight lanes and with one, 50000 atoms: r_c 2^(1/6) 39 and 43, r_c 2.5
+// 104 and 120; 100000 atoms: 56 and 49, 167 and 132.  (The FP64 form, which
+// queues the candidates that pass its FP32 test, keeps eight at every size.)
+constexpr int64_t kCellWide = 65536;
 // The one-launch step loop of small systems (md_run.cuh): kRunLanes lanes per
 // atom; blocks of 128, 256 or 384 threads, two of the largest on an SM (with
 // 80 registers a thread), so that every block of the launch is resident;

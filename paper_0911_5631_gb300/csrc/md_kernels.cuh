@@ -1082,6 +1082,73 @@ __global__ void __launch_bounds__(kBlock) k_cell_forces(Args<P> a) {
     if (__any_sync(0xffffffffu, in && acc.close) && lane == 0) atomicOr(&a.ctr->close_flag, 1);
 }
 
+// The same for large systems in the mixed form, a thread per atom in cell
+// order: with threads enough to fill the device the instructions bound it,
+// and eight lanes spend most of theirs on the ranges of 27 cells, the
+// candidates that a cell does not have and the sums over the lanes.  The sums
+// are integers, so the results are the same bits.  A step of
+// 1M atoms (r_c 2^(1/6), rho 0.8) takes 236 us, 354 with eight lanes per atom and
+// 279 with a thread per atom in the step kernel; with r_c 2.5 666, 1141 and 748.
+// (One candidate loaded ahead: 250 and 744; four: 242 and 654, but 192 against
+// 176 at rho 0.3.)
+template <bool kEnergy>
+__global__ void __launch_bounds__(kBlock) k_cell_forces_wide(Args<Mixed> a) {
+    constexpr int kAhead = 2;  // candidates of a cell loaded before they are used
+    const int64_t s = gtid();
+    AccMixed acc;
+    if (s < a.n) {
+        const float4 ci = __ldg(a.cand + s);
+        const int i = __float_as_int(ci.w), n = (int)a.n;
+        int cx, cy, cz;
+        unpack_cell(a.cell[i], cx, cy, cz);
+        const int xs[3] = {wrap_add(cx, -1, a.G[0]), cx, wrap_add(cx, 1, a.G[0])};
+        int lo[3], hi[3];
+        auto ranges = [&](int r) {  // of the three cells of row r
+            const PencilRow pr = pencil_row(wrap_add(cy, r % 3 - 1, a.G[1]), wrap_add(cz, r / 3 - 1, a.G[2]), a.G);
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const int c = pr.base + xs[k] * pr.stride;
+                lo[k] = __ldg(a.cell_start + c);
+                hi[k] = min(__ldg(a.cell_start + c + 1), n);
+            }
+        };
+        ranges(0);
+        for (int r = 0; r < 9; r++) {
+            int b[3], e[3];
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                b[k] = lo[k];
+                e[k] = hi[k];
+            }
+            if (r < 8) ranges(r + 1);
+            const float sy = -(float)(r % 3 - 1) * a.wf[1], sz = -(float)(r / 3 - 1) * a.wf[2];
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const float sx = -(float)(k - 1) * a.wf[0];
+                for (int t = b[k]; t < e[k]; t += kAhead) {
+                    float4 p[kAhead];
+#pragma unroll
+                    for (int u = 0; u < kAhead; u++)
+                        if (t + u < e[k]) p[u] = __ldg(a.cand + t + u);
+#pragma unroll
+                    for (int u = 0; u < kAhead; u++)
+                        if (t + u < e[k] && t + u != (int)s)
+                            acc.template pair<kEnergy>(a, (ci.x - p[u].x) + sx, (ci.y - p[u].y) + sy,
+                                                       (ci.z - p[u].z) + sz);
+                }
+            }
+        }
+        a.fx[i] = acc.force_x();
+        a.fy[i] = acc.force_y();
+        a.fz[i] = acc.force_z();
+        if constexpr (kEnergy) {
+            a.s_ox[i] = 0.5 * acc.energy();
+            a.s_oy[i] = 0.5 * acc.virial();
+        }
+    }
+    if (__any_sync(0xffffffffu, acc.close) && (threadIdx.x & 31) == 0) atomicOr(&a.ctr->close_flag, 1);
+}
+
 // ---------------------------------------------------------------------------
 // state load
 // ---------------------------------------------------------------------------
@@ -3004,6 +3071,12 @@ KernelTable<P> make_kernel_table() {
     t.step_list_final = (void*)k_step<P, false, true>;
     t.cell_forces = (void*)k_cell_forces<P, false>;
     t.cell_forces_final = (void*)k_cell_forces<P, true>;
+    if constexpr (P::kFp64) {
+        t.cell_forces_wide = t.cell_forces_wide_final = nullptr;
+    } else {
+        t.cell_forces_wide = (void*)k_cell_forces_wide<false>;
+        t.cell_forces_wide_final = (void*)k_cell_forces_wide<true>;
+    }
     t.step_cells = (void*)k_step<P, true, false>;
     t.step_cells_final = (void*)k_step<P, true, true>;
     t.finalize = (void*)k_finalize<P>;

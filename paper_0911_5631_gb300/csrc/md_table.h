@@ -26,6 +26,8 @@ struct KernelTable {
     void* step_list_final;
     void* cell_forces;        // cell-list-only forces, before step_cells
     void* cell_forces_final;  // the same with energies
+    void* cell_forces_wide;   // large systems, mixed form only
+    void* cell_forces_wide_final;
     void* step_cells;
     void* step_cells_final;
     void* finalize;

@@ -526,3 +526,27 @@ def test_cells_only_forces_take_the_pair_coordinate():
             f.append(s.forces())
             s.close()
         assert f[0][0, 0] != 0.0 and np.array_equal(f[0], f[1])
+
+
+# the last size of the cells-only variant with eight lanes per atom and the
+# first ones with a thread per atom (mixed form), cells of one atom and of about
+# ten: forces and sums against the oracle, then steps as graphs and as stream
+# launches
+@pytest.mark.parametrize("n,rho,rc", [(65535, 0.8, RC), (65536, 0.8, RC), (70001, 0.3, RC), (66000, 0.8, 2.5)])
+def test_cells_only_around_the_size_of_a_thread_per_atom(n, rho, rc):
+    pos, vel, L = state(n, rho, 1.0, 65, jitter=0.1)
+    pw = oracle.wrap(pos, L)
+    shift = oracle.wca_shift(rc)
+    f_ref, U, W = oracle.forces_cells(pw, L, oracle_grid(L, rc), rc, shift, threaded=True)
+    out = []
+    for graphs in (True, False):
+        s = md.Simulation(L, n, rc, 0.0, DT, cell_list_only=True, reorder_interval=5, use_graphs=graphs)
+        s.set_state(pos, vel)
+        m = s.measure()
+        assert rel_rms(s.forces(), f_ref) <= FORCE_TOL["mixed"]
+        assert m["pe"] == pytest.approx(U, rel=10 * FORCE_TOL["mixed"])
+        assert m["virial"] == pytest.approx(W, rel=10 * FORCE_TOL["mixed"])
+        s.step(12)
+        out.append(s.get_state() + (s.forces(),))
+        s.close()
+    assert all(np.array_equal(x, y) for x, y in zip(*out))
