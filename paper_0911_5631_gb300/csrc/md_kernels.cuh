@@ -1381,12 +1381,16 @@ __device__ __forceinline__ bool sorts_cells(int reorder) {
     return P::kFp64 || reorder;
 }
 
-// The candidate that an atom is to the neighbour search (and, in the mixed
-// cells-only variant, to the forces): its pair coordinate, which the binning has
-// just written, and its storage index.  (pb alone is the same number but for an
-// offset that FP32 rounds onto half a unit of pb's last place.)
+// The candidate that an atom is to the neighbour search and, in the cells-only
+// variant, to the forces: its FP32 coordinates and storage index.  The forces
+// take the pair coordinate, which the binning has just written; for a search,
+// whose margin is far wider, the offset pb serves, with 4 bytes less per atom to
+// read (the two differ where FP32 rounds the rest of an offset onto half a unit
+// of pb's last place).
 __device__ __forceinline__ float4 candidate(const Args<Mixed>& a, int64_t i, int index, int parity) {
-    const float4 p = (parity ? a.pB : a.pA)[i];
+    float4 p;
+    if (a.cell_list_only) p = (parity ? a.pB : a.pA)[i];
+    else p = make_float4(a.pbx[i], a.pby[i], a.pbz[i], 0.0f);
     return make_float4(p.x, p.y, p.z, __int_as_float(index));
 }
 
